@@ -357,7 +357,7 @@ bool pack(const bpdc_graph_s &g, const Variant &v, Packed &P)
             P.l_cols[(size_t)j * kw + (k >> 5)] |= 1u << (k & 31);
             P.l_pos[(size_t)lay.pos_of_var[j] * kw + (k >> 5)] |= 1u << (k & 31);
         }
-    P.thr.resize(N);
+    P.thr.assign((size_t)P.NW * 32, 0);
     for (int j = 0; j < N; ++j) P.thr[j] = (uint32_t)std::floor(g.priors[j] * 4294967296.0);
     return true;
 }
@@ -411,20 +411,38 @@ int plan_and_upload(bpdc_graph_s *g, int want_G, int want_id = -1)
     const size_t o_chkw = put(blob, P.chk_word), o_tab = put(blob, P.chk_tab);
     const size_t o_dptr = put(blob, P.d_ptr), o_dent = put(blob, P.d_ent), o_l = put(blob, P.l_pos);
     const size_t o_dcol = put(blob, P.d_col), o_lcol = put(blob, P.l_cols), o_pcol = put(blob, P.pos_col);
-    const size_t o_hptr = put(blob, g->H.ptr), o_hcol = put(blob, g->H.col), o_thr = put(blob, P.thr);
+    const size_t o_hptr = put(blob, g->H.ptr), o_thr = put(blob, P.thr);
     // column view of H and priors by column (weighted BP)
-    std::vector<int32_t> cptr(g->H.cols + 1, 0), cedge(g->H.col.size());
+    std::vector<int32_t> cptr(g->H.cols + 1, 0), cedge(g->H.col.size()), cchk(g->H.col.size());
     std::vector<float> lamc(g->H.cols);
     for (int32_t c : g->H.col) cptr[c + 1]++;
     for (int j = 0; j < g->H.cols; ++j) cptr[j + 1] += cptr[j];
     {
         std::vector<int32_t> fill(cptr.begin(), cptr.end() - 1);
         for (int i = 0; i < g->H.rows; ++i)
-            for (int a = g->H.ptr[i]; a < g->H.ptr[i + 1]; ++a) cedge[fill[g->H.col[a]]++] = a;
+            for (int a = g->H.ptr[i]; a < g->H.ptr[i + 1]; ++a) {
+                const int x = fill[g->H.col[a]]++;
+                cedge[x] = a;
+                cchk[x] = i;
+            }
         for (int j = 0; j < g->H.cols; ++j)
             lamc[j] = (float)std::log((1.0 - g->priors[j]) / g->priors[j]);
     }
     const size_t o_cptr = put(blob, cptr), o_cedge = put(blob, cedge), o_lamc = put(blob, lamc);
+    // rows of H and L as bit masks over the columns (sampler, narrow graphs)
+    std::vector<uint32_t> rmask;
+    if (P.NW <= kSampleMaskWords && P.MW + P.KW <= 32) {
+        const size_t words = (size_t)(P.NW + 3) / 4 * 4;
+        rmask.assign((size_t)(P.MW + P.KW) * 32 * words, 0);
+        auto fill = [&](const HostCsr &m, size_t r0) {
+            for (int i = 0; i < m.rows; ++i)
+                for (int a = m.ptr[i]; a < m.ptr[i + 1]; ++a)
+                    rmask[(r0 + i) * words + (m.col[a] >> 5)] |= 1u << (m.col[a] & 31);
+        };
+        fill(g->H, 0);
+        fill(g->L, (size_t)P.MW * 32);
+    }
+    const size_t o_rmask = put(blob, rmask), o_cchk = put(blob, cchk);
     const size_t o_wts = put(blob, P.wts);
     const size_t o_err = put(blob, std::vector<int32_t>(4, 0));
     void *arena = nullptr;
@@ -462,7 +480,8 @@ int plan_and_upload(bpdc_graph_s *g, int want_G, int want_id = -1)
     d.l_col = (const uint32_t *)(base + o_lcol);
     d.pos_col = (const int32_t *)(base + o_pcol);
     d.h_ptr = (const int32_t *)(base + o_hptr);
-    d.h_col = (const int32_t *)(base + o_hcol);
+    d.row_mask = (const uint4 *)(base + o_rmask);
+    d.c_chk = (const int32_t *)(base + o_cchk);
     d.thr = (const uint32_t *)(base + o_thr);
     d.c_ptr = (const int32_t *)(base + o_cptr);
     d.c_edge = (const int32_t *)(base + o_cedge);

@@ -14,6 +14,9 @@ constexpr float kLlrCap = 1e30f;
 constexpr uint16_t kNoEdge = 0xFFFF;
 // Limits of the compiled kernel variants.
 constexpr int kMaxDRowWeight = 64;
+// The sampler keeps a shot in registers up to this many error words, with the
+// rows of H and L as bit masks.
+constexpr int kSampleMaskWords = 8;
 
 // Message slots per variable pass.  A variant's profile holds 3 bits per pass
 // (pass p in bits 3p .. 3p+2, a non-increasing sequence, up to 21 passes):
@@ -86,11 +89,13 @@ struct DevGraph {
     const uint32_t *l_bits;      // [pv*G][KW] columns of L by variable position
     const uint32_t *l_col;       // [N][KW] columns of L by column index (sampler)
     const int32_t *pos_col;      // [pv*G] column of the variable at each position (-1: none)
-    const int32_t *h_ptr;        // [M+1] rows of H (sampler)
-    const int32_t *h_col;        // [E]
-    const uint32_t *thr;         // [N] floor(p * 2^32) (sampler)
+    const int32_t *h_ptr;        // [M+1] rows of H (weighted BP)
+    const uint4 *row_mask;       // [(MW+KW)*32][ceil(NW/4)] rows of H, then of L, as bit masks, zero-padded to
+                                 // 16 bytes (sampler's narrow form; else empty)
+    const uint32_t *thr;         // [NW*32] floor(p * 2^32), 0 past N (sampler)
     const int32_t *c_ptr;        // [N+1] columns of H: edges of variable j are c_edge[c_ptr[j] .. c_ptr[j+1])
     const int32_t *c_edge;       // [E] edge ids (CSR order of H) by column, ascending check
+    const int32_t *c_chk;        // [E] check of each edge by column, as c_edge (sampler)
     const float *lam_col;        // [N] prior LLR by column (weighted BP)
     int32_t *err_flag;           // latched device error code
 #ifdef BPDC_CHECKS

@@ -1168,48 +1168,6 @@ __global__ void cut_select_kernel(DevGraph g, int64_t B, const float *post, uint
     }
 }
 
-// Seeded sampler: errors, syndromes e H^T and observables e L^T, one block per shot.
-__global__ void sample_kernel(DevGraph g, int64_t B, uint64_t seed, uint64_t shot_offset,
-                              uint32_t *syn, uint32_t *obs, uint32_t *err)
-{
-    extern __shared__ uint32_t sm[];
-    uint32_t *eb = sm, *sb = sm + g.NW, *ob = sb + g.MW;
-    const int nw = g.NW + g.MW + g.KW;
-    for (int64_t b = blockIdx.x; b < B; b += gridDim.x) {
-        for (int x = threadIdx.x; x < nw; x += blockDim.x) sm[x] = 0;
-        __syncthreads();
-        const uint64_t gs = shot_offset + (uint64_t)b;
-        for (int j = threadIdx.x; j < g.N; j += blockDim.x) {
-            const uint64_t h = splitmix64(seed, gs * (uint64_t)g.N + (uint64_t)j);
-            if ((uint32_t)(h >> 32) < __ldg(g.thr + j)) atomicOr(eb + (j >> 5), 1u << (j & 31));
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < g.M; i += blockDim.x) {
-            uint32_t par = 0;
-            for (int a = __ldg(g.h_ptr + i); a < __ldg(g.h_ptr + i + 1); ++a) {
-                const int c = __ldg(g.h_col + a);
-                par ^= (eb[c >> 5] >> (c & 31)) & 1u;
-            }
-            if (par) atomicOr(sb + (i >> 5), 1u << (i & 31));
-        }
-        for (int j = threadIdx.x; j < g.N; j += blockDim.x) {
-            if ((eb[j >> 5] >> (j & 31)) & 1u) {
-                for (int x = 0; x < g.KW; ++x) {
-                    const uint32_t v = __ldg(g.l_col + (size_t)j * g.KW + x);
-                    if (v) atomicXor(ob + x, v);
-                }
-            }
-        }
-        __syncthreads();
-        for (int x = threadIdx.x; x < g.MW; x += blockDim.x) syn[(size_t)b * g.MW + x] = sb[x];
-        if (obs)
-            for (int x = threadIdx.x; x < g.KW; x += blockDim.x) obs[(size_t)b * g.KW + x] = ob[x];
-        if (err)
-            for (int x = threadIdx.x; x < g.NW; x += blockDim.x) err[(size_t)b * g.NW + x] = eb[x];
-        __syncthreads();
-    }
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -1422,21 +1380,6 @@ cudaError_t launch_cut_select(const DevGraph &g, int64_t B, const float *post, u
     if (B <= 0) return cudaSuccess;
     const int grid = (int)(B < 65536 ? B : 65536);
     cut_select_kernel<<<grid, 256, g.NW * 4, s>>>(g, B, post, shot_offset, cut_out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sample(const DevGraph &g, int64_t B, uint64_t seed, uint64_t shot_offset,
-                          uint32_t *syn, uint32_t *obs, uint32_t *err, cudaStream_t s)
-{
-    if (B <= 0) return cudaSuccess;
-    const int smem = (g.NW + g.MW + g.KW) * 4;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute((const void *)sample_kernel,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-    }
-    const int grid = (int)(B < 152 * 16 ? B : 152 * 16);
-    sample_kernel<<<grid, 256, smem, s>>>(g, B, seed, shot_offset, syn, obs, err);
     return cudaGetLastError();
 }
 
