@@ -341,11 +341,12 @@ int bpdc_measure_smem_peak(int32_t device, int32_t reps, double *bytes_per_secon
  *            phi(sum_{e' in N(i), e' != e} phi(max(|q_e'(t)|, 1e-6))),   phi(x) = -log tanh(x/2)
  *   L_j(t) = lambda_j + sum_{e in M(j)} r_e(t)
  * Unit weights and a large clip give the decoder's product-sum BP.  Graphs
- * need row weights 2..16 and column weights <= 8.  The forward keeps the q of
- * iterations 0, k, 2k, ... (k = ckpt_every) in the caller's workspace; the
- * backward recomputes each k-iteration segment from them, so both calls must
- * get the same workspace, weights, syndromes, T, clip and ckpt_every, with the
- * forward first.  Calls are stream-ordered and asynchronous.  Errors:
+ * need row weights 2..16 and column weights <= 8.  The forward keeps what the
+ * backward needs of every iteration in the caller's workspace, so both calls
+ * must get the same workspace, weights, syndromes, T, clip and ckpt_every, with
+ * the forward first (the backward leaves it as it was and may be called again).
+ * ckpt_every (an interval of iterations) enters the size of the workspace only;
+ * no result depends on it.  Calls are stream-ordered and asynchronous.  Errors:
  * BPDC_ERR_INVALID_ARG (NULL buffers, T outside [1, 1000], ckpt_every
  * outside [1, T], clip outside (0, 30], workspace too small),
  * BPDC_ERR_UNSUPPORTED (row/column weights, or more edges than the adjoint's

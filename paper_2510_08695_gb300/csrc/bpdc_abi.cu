@@ -413,7 +413,8 @@ int plan_and_upload(bpdc_graph_s *g, int want_G, int want_id = -1)
     const size_t o_dcol = put(blob, P.d_col), o_lcol = put(blob, P.l_cols), o_pcol = put(blob, P.pos_col);
     const size_t o_hptr = put(blob, g->H.ptr), o_thr = put(blob, P.thr);
     // column view of H and priors by column (weighted BP)
-    std::vector<int32_t> cptr(g->H.cols + 1, 0), cedge(g->H.col.size()), cchk(g->H.col.size());
+    std::vector<int32_t> cptr(g->H.cols + 1, 0), cchk(g->H.col.size());
+    std::vector<uint16_t> cedget;   // weighted BP: at most kWbpMaxCol edges of a column and 65535 in all
     std::vector<float> lamc(g->H.cols);
     for (int32_t c : g->H.col) cptr[c + 1]++;
     for (int j = 0; j < g->H.cols; ++j) cptr[j + 1] += cptr[j];
@@ -421,14 +422,16 @@ int plan_and_upload(bpdc_graph_s *g, int want_G, int want_id = -1)
         std::vector<int32_t> fill(cptr.begin(), cptr.end() - 1);
         for (int i = 0; i < g->H.rows; ++i)
             for (int a = g->H.ptr[i]; a < g->H.ptr[i + 1]; ++a) {
-                const int x = fill[g->H.col[a]]++;
-                cedge[x] = a;
+                const int c = g->H.col[a], x = fill[c]++, m = x - cptr[c];
                 cchk[x] = i;
+                if (m >= kWbpMaxCol || a >= 0xFFFF) continue;
+                if (cedget.size() < (size_t)(m + 1) * g->H.cols) cedget.resize((size_t)(m + 1) * g->H.cols, 0xFFFF);
+                cedget[(size_t)m * g->H.cols + c] = (uint16_t)a;
             }
         for (int j = 0; j < g->H.cols; ++j)
             lamc[j] = (float)std::log((1.0 - g->priors[j]) / g->priors[j]);
     }
-    const size_t o_cptr = put(blob, cptr), o_cedge = put(blob, cedge), o_lamc = put(blob, lamc);
+    const size_t o_cptr = put(blob, cptr), o_cedge = put(blob, cedget), o_lamc = put(blob, lamc);
     // rows of H and L as bit masks over the columns (sampler, narrow graphs)
     std::vector<uint32_t> rmask;
     if (P.NW <= kSampleMaskWords && P.MW + P.KW <= 32) {
@@ -484,7 +487,7 @@ int plan_and_upload(bpdc_graph_s *g, int want_G, int want_id = -1)
     d.c_chk = (const int32_t *)(base + o_cchk);
     d.thr = (const uint32_t *)(base + o_thr);
     d.c_ptr = (const int32_t *)(base + o_cptr);
-    d.c_edge = (const int32_t *)(base + o_cedge);
+    d.c_edget = (const uint16_t *)(base + o_cedge);
     d.lam_col = (const float *)(base + o_lamc);
     d.wts = P.wts.empty() ? nullptr : (const float *)(base + o_wts);
     d.w_T = P.wts.empty() ? 0 : g->w_T;
@@ -1221,12 +1224,11 @@ static int wbp_prepare(bpdc_graph_t g, int64_t B, const uint32_t *syndromes, con
     bpdc_wbp_workspace_size(g, B, T, ckpt_every, &need);
     if (B > 0 && (!workspace || workspace_bytes < need))
         return fail(BPDC_ERR_INVALID_ARG, "workspace of %zu bytes needed", need);
-    const size_t nck = (size_t)B * ((T + ckpt_every - 1) / ckpt_every) * E;
     a = WbpArgs{};
-    a.B = B; a.E = E; a.T = T; a.k = ckpt_every; a.clip = clip;
+    a.B = B; a.E = E; a.T = T; a.rm = rmax; a.cm = cmax; a.clip = clip;
     a.syn = syndromes; a.W = weights;
-    a.ckpt = (float *)workspace;
-    a.part = (float *)workspace + ((nck + 63) & ~(size_t)63);
+    a.part = (float *)workspace;
+    a.S = (float *)workspace + need / sizeof(float) - (size_t)B * T * E;
     return BPDC_OK;
 }
 

@@ -93,9 +93,10 @@ struct DevGraph {
     const uint4 *row_mask;       // [(MW+KW)*32][ceil(NW/4)] rows of H, then of L, as bit masks, zero-padded to
                                  // 16 bytes (sampler's narrow form; else empty)
     const uint32_t *thr;         // [NW*32] floor(p * 2^32), 0 past N (sampler)
-    const int32_t *c_ptr;        // [N+1] columns of H: edges of variable j are c_edge[c_ptr[j] .. c_ptr[j+1])
-    const int32_t *c_edge;       // [E] edge ids (CSR order of H) by column, ascending check
-    const int32_t *c_chk;        // [E] check of each edge by column, as c_edge (sampler)
+    const int32_t *c_ptr;        // [N+1] columns of H: checks of column j are c_chk[c_ptr[j] .. c_ptr[j+1])
+    const int32_t *c_chk;        // [E] check of each edge by column, ascending (sampler)
+    const uint16_t *c_edget;     // [column weight][N] edge (CSR order of H) m of column j at m * N + j, 0xFFFF
+                                 // past its weight (weighted BP)
     const float *lam_col;        // [N] prior LLR by column (weighted BP)
     int32_t *err_flag;           // latched device error code
 #ifdef BPDC_CHECKS
@@ -191,16 +192,16 @@ constexpr int kWbpMaxCol = 8;
 constexpr size_t kMaxWbpSmem = 227 * 1024;
 struct WbpArgs {
     int64_t B;
-    int E, T, k;                 // edges, iterations, checkpoint interval
+    int E, T;                    // edges, iterations
+    int rm, cm;                  // largest row and column weight
     float clip;                  // |q| <= clip
     const uint32_t *syn;         // [B][MW]
     const float *W;              // [2][T][E]
     float *post;                 // [B][T][N] or null
-    float *ckpt;                 // [B][ceil(T/k)][E] q of iterations 0, k, 2k, ...
+    float *S;                    // [B][T][E] sum of phi over the other edges of the check, with r's sign
     const float *gpost;          // [B][T][N] adjoint of the posteriors (backward)
-    float *part;                 // [B][2][T][E] per-shot gradient partials (backward)
+    float *part;                 // [blocks][2: hi, lo][2][T][E] partial gradients (backward)
 };
-size_t wbp_smem_forward(int E, int warps);
 size_t wbp_smem_backward(int E, int k, int warps);
 cudaError_t launch_wbp_forward(const DevGraph &g, const WbpArgs &a, cudaStream_t s);
 cudaError_t launch_wbp_backward(const DevGraph &g, const WbpArgs &a, float *grad_w, cudaStream_t s);

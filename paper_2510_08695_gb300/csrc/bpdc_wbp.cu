@@ -11,17 +11,33 @@
 // phi(x) = -log tanh(x/2) (Sec. II.C.1's product-sum rule in log form).  With
 // unit weights and no clipping this is the decoder's flooding product-sum BP.
 //
-// Forward: one warp per shot, q and r of the shot in shared memory; the q of
-// every k-th iteration is checkpointed to global memory.  Adjoint: per shot,
-// segments of k iterations are recomputed from their checkpoint into shared
-// memory and then run backwards; with phi'(x) = -1/sinh(x),
-//   d r_e / d q_e' = wc_e s_e sgn(q_e') / (sinh(S_e) sinh(|q_e'|)),
-// so the adjoint of q_e' is sgn(q_e') / sinh(|q_e'|) times the sum over the
-// other edges e of the check of rbar_e wc_e s_e / sinh(S_e) (prefix and suffix
-// sums, no subtraction).  Every shot writes its own gradient partials; a
-// second kernel sums them over shots in a fixed order (deterministic).
+// Bound by instruction issue: phi (log1p of a quotient by expm1) and 1 / sinh take
+// some 60 instructions each and are evaluated twice per edge and iteration in the
+// forward, three times in the adjoint.  So those run with one lane per edge (432
+// edges: 14 passes of a warp, 96 % of the lanes; a lane per check would keep 72 of
+// 96), and only the short sums over a check or a variable run with a lane per
+// check or variable, in place over one value per edge in shared memory.
+//
+// A team of G threads decodes a shot: 64 when there are enough shots, else 256.
+// The forward saves S of every iteration (with the outgoing sign) in the
+// workspace: r(t) = wc phi(S) and then q(t+1) follow from it, so the adjoint
+// neither keeps a segment of q and r in shared memory (which left 8 warps on an
+// SM) nor evaluates phi(|q|) again.  Every operation is the one the definition
+// gives, in one fixed order, so gradients of long unrolled runs, which amplify
+// rounding, do not depend on the launch.
+//
+// Gradients are summed over shots in a fixed order: the shots of a block (4 to 8)
+// in shared memory at each iteration, the blocks' sums by a second kernel.  Sums
+// are pairs hi + lo of floats (error-free two-sum): FP64 adds run at a 64th of the
+// FP32 rate here, and a store of every shot's gradients was 283 MB a call.
+//
+// BB[[144,12,12]], T = 20, 4096 shots: forward 545 -> 299 us (issue 79 %), adjoint
+// 2540 -> 503 us (11 900 -> 5050 warp instructions per shot and iteration, issue
+// 70 %), sum of the gradients 790 -> 25 us.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cmath>
 #include <cstdint>
 
 #include "bpdc_internal.h"
@@ -30,6 +46,9 @@ namespace bpdc {
 namespace {
 
 constexpr float kQmin = 1e-6f;
+constexpr int kNoEdge16 = 0xFFFF;
+// Most edges (as ever: the message arrays of eight shots fit a block's memory).
+constexpr int kWbpMaxEdges = (int)(kMaxWbpSmem / (8 * 2 * sizeof(float)));
 
 __device__ __forceinline__ float wphi(float x) { return log1pf(2.0f / expm1f(x)); }
 
@@ -38,298 +57,367 @@ __device__ __forceinline__ float inv_sinh(float x) { return 2.0f * expf(-x) / -e
 
 __device__ __forceinline__ uint32_t syn_bit(const uint32_t *sy, int i) { return (__ldg(sy + (i >> 5)) >> (i & 31)) & 1u; }
 
-// q(t) from r(t-1): lanes over variables
-__device__ void wbp_var_phase(const DevGraph &g, const float *r, float *q, const float *wv, float clip, int lane)
+__device__ __forceinline__ float with_sign(float mag, bool neg)
 {
-    for (int j = lane; j < g.N; j += 32) {
-        const int c0 = __ldg(g.c_ptr + j), d = __ldg(g.c_ptr + j + 1) - c0;
-        const float lam = __ldg(g.lam_col + j);
-        int ee[kWbpMaxCol];
-        float rr[kWbpMaxCol], pre[kWbpMaxCol + 1];
-        pre[0] = 0.0f;
+    return __uint_as_float(__float_as_uint(mag) | (neg ? 0x80000000u : 0u));
+}
+__device__ __forceinline__ bool sign_of(float x) { return (__float_as_uint(x) >> 31) != 0u; }
+
+// The G threads that work on a shot; named barrier 1 + index of the shot in the block.
+template <int G>
+__device__ __forceinline__ void team_sync(int team)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(G) : "memory");
+}
+
+// A sum kept as hi + lo: lo collects the exact rounding errors of hi (two-sum),
+// which carries some 48 bits; with an overflow or a NaN only hi counts.
+struct Sum2 {
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void add(float x)
+    {
+        const float s = hi + x, b = s - hi;
+        lo += (hi - (s - b)) + (x - b);
+        hi = s;
+    }
+    __device__ __forceinline__ float value() const { return isfinite(hi) ? hi + lo : hi; }
+};
+
+// In place over the edges of every variable (lanes over variables; m-th edge of
+// variable j in c_edget[m * N + j]): out(j, base, pre_m + suf_m) with pre_m / suf_m
+// the sums of the values before / after edge m, and total(j, values) per variable.
+template <int G, int CM, typename Base, typename Total>
+__device__ __forceinline__ void var_phase(const DevGraph &g, float *x, int u, int cm, bool write, Base base, Total total)
+{
+    for (int j = u; j < g.N; j += G) {
+        int ee[CM];
+        float v[CM], pre[CM];
+        float sum = 0.0f;
 #pragma unroll
-        for (int m = 0; m < kWbpMaxCol; ++m) {
-            ee[m] = m < d ? __ldg(g.c_edge + c0 + m) : 0;
-            rr[m] = m < d ? r[ee[m]] : 0.0f;
-            pre[m + 1] = pre[m] + rr[m];
+        for (int m = 0; m < CM; ++m) {
+            ee[m] = kNoEdge16;
+            v[m] = 0.0f;
+            if (m < cm) {
+                ee[m] = __ldg(g.c_edget + m * g.N + j);
+                if (ee[m] != kNoEdge16) v[m] = x[ee[m]];
+            }
+            pre[m] = sum;
+            sum += v[m];
         }
+        const float b = base(j);
+        total(j, b, v);
+        if (!write) continue;
         float suf = 0.0f;
 #pragma unroll
-        for (int m = kWbpMaxCol - 1; m >= 0; --m) {
-            if (m < d) {
-                const float z = __ldg(wv + ee[m]) * (lam + (pre[m] + suf));
-                q[ee[m]] = fminf(fmaxf(z, -clip), clip);
-                suf += rr[m];
-            }
+        for (int m = CM - 1; m >= 0; --m) {
+            if (ee[m] != kNoEdge16) x[ee[m]] = b + (pre[m] + suf);
+            suf += v[m];
         }
     }
 }
 
-// r(t) from q(t): lanes over checks
-__device__ void wbp_chk_phase(const DevGraph &g, const float *q, float *r, const float *wc, const uint32_t *sy,
-                              int lane)
-{
-    for (int i = lane; i < g.M; i += 32) {
-        const int e0 = __ldg(g.h_ptr + i), d = __ldg(g.h_ptr + i + 1) - e0;
-        float f[kWbpMaxRow], suf[kWbpMaxRow + 1];
-        uint32_t negs = 0, par = syn_bit(sy, i);
-#pragma unroll
-        for (int k = 0; k < kWbpMaxRow; ++k) {
-            f[k] = 0.0f;
-            if (k < d) {
-                const float x = q[e0 + k];
-                f[k] = wphi(fmaxf(fabsf(x), kQmin));
-                const uint32_t ng = x < 0.0f ? 1u : 0u;
-                negs |= ng << k;
-                par ^= ng;
-            }
-        }
-        suf[kWbpMaxRow] = 0.0f;
-#pragma unroll
-        for (int k = kWbpMaxRow - 1; k >= 0; --k) suf[k] = suf[k + 1] + f[k];
-        float pre = 0.0f;
-#pragma unroll
-        for (int k = 0; k < kWbpMaxRow; ++k) {
-            if (k < d) {
-                const float c = wphi(pre + suf[k + 1]);
-                const bool neg = ((par ^ (negs >> k)) & 1u) != 0;
-                r[e0 + k] = __ldg(wc + e0 + k) * (neg ? -c : c);
-                pre += f[k];
-            }
-        }
-    }
-}
-
-__global__ void wbp_forward_kernel(DevGraph g, WbpArgs a)
+template <int G, int CM, int RM>
+__global__ void __launch_bounds__(G == 64 ? 512 : 1024, G == 64 ? 4 : 2) wbp_forward_kernel(DevGraph g, WbpArgs a)
 {
     extern __shared__ float sm[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-    const int E = a.E;
-    float *r = sm + (size_t)warp * 2 * E, *q = r + E;
-    const int nseg = (a.T + a.k - 1) / a.k;
-    for (int64_t b = (int64_t)blockIdx.x * wpb + warp; b < a.B; b += (int64_t)gridDim.x * wpb) {
-        const uint32_t *sy = a.syn + b * g.MW;
-        for (int e = lane; e < E; e += 32) r[e] = 0.0f;
-        __syncwarp();
-        for (int t = 0; t < a.T; ++t) {
-            wbp_var_phase(g, r, q, a.W + (size_t)(a.T + t) * E, a.clip, lane);
-            __syncwarp();
-            if (a.ckpt && t % a.k == 0) {
-                float *ck = a.ckpt + ((size_t)b * nseg + t / a.k) * E;
-                for (int e = lane; e < E; e += 32) ck[e] = q[e];
-            }
-            wbp_chk_phase(g, q, r, a.W + (size_t)t * E, sy, lane);
-            __syncwarp();
-            if (a.post) {
-                float *pr = a.post + ((size_t)b * a.T + t) * g.N;
-                for (int j = lane; j < g.N; j += 32) {
-                    const int c0 = __ldg(g.c_ptr + j), c1 = __ldg(g.c_ptr + j + 1);
-                    float L = __ldg(g.lam_col + j);
-                    for (int c = c0; c < c1; ++c) L += r[__ldg(g.c_edge + c)];
-                    pr[j] = L;
-                }
-            }
-        }
-        __syncwarp();
-    }
-}
-
-__global__ void wbp_backward_kernel(DevGraph g, WbpArgs a)
-{
-    extern __shared__ float sm[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-    const int E = a.E, T = a.T, K = a.k;
-    float *Qs = sm + (size_t)warp * (2 * K + 2) * E;   // q(t0 .. t0+K-1) of the current segment
-    float *Rs = Qs + (size_t)K * E;                     // r(t0 .. t0+K-1)
-    float *QB = Rs + (size_t)K * E;                     // adjoint of q(t+1), then of q(t)
-    float *RB = QB + E;                                 // adjoint of r(t)
-    const int nseg = (T + K - 1) / K;
+    const int team = threadIdx.x / G, u = threadIdx.x % G, W = blockDim.x / G;
+    const int E = a.E, T = a.T;
+    float *x = sm + (size_t)team * E;   // per edge: r, then lambda + sum r, phi(|q|), S, r again
     const float clip = a.clip;
-    for (int64_t b = (int64_t)blockIdx.x * wpb + warp; b < a.B; b += (int64_t)gridDim.x * wpb) {
+    for (int64_t b = (int64_t)blockIdx.x * W + team; b < a.B; b += (int64_t)gridDim.x * W) {
         const uint32_t *sy = a.syn + b * g.MW;
-        const float *gp = a.gpost + (size_t)b * T * g.N;
-        float *part = a.part + (size_t)b * 2 * T * E;   // [2][T][E] partials of this shot
-        for (int e = lane; e < E; e += 32) QB[e] = 0.0f;
-        for (int seg = nseg - 1; seg >= 0; --seg) {
-            const int t0 = seg * K, nt = min(K, T - t0);
-            const float *ck = a.ckpt + ((size_t)b * nseg + seg) * E;
-            for (int e = lane; e < E; e += 32) Qs[e] = ck[e];
-            __syncwarp();
-            for (int u = 0; u < nt; ++u) {   // recompute the segment
-                wbp_chk_phase(g, Qs + (size_t)u * E, Rs + (size_t)u * E, a.W + (size_t)(t0 + u) * E, sy, lane);
-                __syncwarp();
-                if (u + 1 < nt) {
-                    wbp_var_phase(g, Rs + (size_t)u * E, Qs + (size_t)(u + 1) * E, a.W + (size_t)(T + t0 + u + 1) * E,
-                                  clip, lane);
-                    __syncwarp();
+        float *post = a.post ? a.post + (size_t)b * T * g.N : nullptr;
+        float *save = a.S + (size_t)b * T * E;
+        for (int e = u; e < E; e += G) x[e] = 0.0f;
+        team_sync<G>(team);
+        for (int t = 0; t <= T; ++t) {
+            // posteriors of iteration t-1 and lambda + the other r of iteration t
+            var_phase<G, CM>(
+                g, x, u, a.cm, t < T, [&](int j) { return __ldg(g.lam_col + j); },
+                [&](int j, float lam, const float (&r)[CM]) {
+                    if (!post || t == 0) return;
+                    float L = lam;
+#pragma unroll
+                    for (int m = 0; m < CM; ++m) L += r[m];
+                    post[(size_t)(t - 1) * g.N + j] = L;
+                });
+            if (t == T) break;
+            team_sync<G>(team);
+            const float *wv = a.W + (size_t)(T + t) * E, *wc = a.W + (size_t)t * E;
+            for (int e = u; e < E; e += G) {
+                const float q = fminf(fmaxf(__ldg(wv + e) * x[e], -clip), clip);
+                x[e] = with_sign(wphi(fmaxf(fabsf(q), kQmin)), q < 0.0f);
+            }
+            team_sync<G>(team);
+            for (int i = u; i < g.M; i += G) {
+                const int e0 = __ldg(g.h_ptr + i), d = __ldg(g.h_ptr + i + 1) - e0;
+                float f[RM], suf[RM + 1];
+                uint32_t negs = 0, par = syn_bit(sy, i);
+#pragma unroll
+                for (int k = 0; k < RM; ++k) {
+                    f[k] = 0.0f;
+                    if (k < d) {
+                        const float v = x[e0 + k];
+                        f[k] = fabsf(v);
+                        const uint32_t ng = sign_of(v) ? 1u : 0u;
+                        negs |= ng << k;
+                        par ^= ng;
+                    }
+                }
+                suf[RM] = 0.0f;
+#pragma unroll
+                for (int k = RM - 1; k >= 0; --k) suf[k] = suf[k + 1] + f[k];
+                float pre = 0.0f;
+#pragma unroll
+                for (int k = 0; k < RM; ++k) {
+                    if (k < d) {
+                        x[e0 + k] = with_sign(pre + suf[k + 1], ((par ^ (negs >> k)) & 1u) != 0);
+                        pre += f[k];
+                    }
                 }
             }
-            for (int u = nt - 1; u >= 0; --u) {
-                const int t = t0 + u;
-                const float *rt = Rs + (size_t)u * E;
-                const float *qt = Qs + (size_t)u * E;
-                // (1) adjoint of r(t): posterior L(t) and, through q(t+1), the
-                // variable updates of iteration t+1 (also their wv gradient)
-                const bool next = t + 1 < T;
-                const float *wv1 = a.W + (size_t)(T + t + 1) * E;
-                for (int j = lane; j < g.N; j += 32) {
-                    const int c0 = __ldg(g.c_ptr + j), d = __ldg(g.c_ptr + j + 1) - c0;
-                    const float lam = __ldg(g.lam_col + j);
-                    const float gl = gp[(size_t)t * g.N + j];
-                    int ee[kWbpMaxCol];
-                    float rr[kWbpMaxCol], ab[kWbpMaxCol], pre[kWbpMaxCol + 1];
-                    pre[0] = 0.0f;
+            team_sync<G>(team);
+            for (int e = u; e < E; e += G) {
+                const float sv = x[e], c = wphi(fabsf(sv));
+                save[(size_t)t * E + e] = sv;
+                x[e] = __ldg(wc + e) * (sign_of(sv) ? -c : c);
+            }
+            team_sync<G>(team);
+        }
+        team_sync<G>(team);
+    }
+}
+
+template <int G, int CM, int RM>
+__global__ void __launch_bounds__(G == 64 ? 512 : 1024, G == 64 ? 4 : 2) wbp_backward_kernel(DevGraph g, WbpArgs a, float *grad_w)
+{
+    extern __shared__ float sm[];
+    const int team = threadIdx.x / G, u = threadIdx.x % G, W = blockDim.x / G;
+    const int E = a.E, T = a.T;
+    const size_t nw = (size_t)2 * T * E;
+    // per shot and edge: adjoint chain, r(t-1) then lambda + the others then the wv
+    // gradient, c(t) = phi(S(t)), the wc gradient
+    float *x = sm + (size_t)team * 4 * E, *r = x + E, *cc = r + E, *pc = cc + E;
+    const float clip = a.clip;
+    float *part = a.part + (size_t)blockIdx.x * 2 * nw;
+    const bool direct = (int64_t)W >= a.B;   // one block, one round: the sum is the result
+    for (int64_t base = (int64_t)blockIdx.x * W; base < a.B; base += (int64_t)gridDim.x * W) {
+        const int64_t b = base + team;
+        const bool on = b < a.B;
+        const int shots = (int)(a.B - base < W ? a.B - base : W);
+        const float *gp = a.gpost + (size_t)b * T * g.N, *S = a.S + (size_t)b * T * E;
+        if (on) {
+            for (int e = u; e < E; e += G) {
+                x[e] = 0.0f;
+                cc[e] = wphi(fabsf(__ldg(S + (size_t)(T - 1) * E + e)));
+            }
+            team_sync<G>(team);
+        }
+        for (int t = T - 1; t >= 0; --t) {
+            // adjoint of r(t): the posterior L(t) and, through q(t+1), the other edges
+            if (on)
+                var_phase<G, CM>(
+                    g, x, u, a.cm, true, [&](int j) { return __ldg(gp + (size_t)t * g.N + j); },
+                    [](int, float, const float (&)[CM]) {});
+            __syncthreads();   // and the previous iteration's sums have been taken
+            if (on) {
+                const float *wc = a.W + (size_t)t * E, *St = S + (size_t)t * E;
+                for (int e = u; e < E; e += G) {
+                    const float rb = x[e], sv = __ldg(St + e);
+                    const float s = sign_of(sv) ? -1.0f : 1.0f;
+                    pc[e] = rb * s * cc[e];
+                    x[e] = rb * __ldg(wc + e) * s * inv_sinh(fabsf(sv));
+                    if (t > 0) {
+                        const float s1 = __ldg(St - E + e), c1 = wphi(fabsf(s1));
+                        cc[e] = c1;
+                        r[e] = __ldg(wc - E + e) * (sign_of(s1) ? -c1 : c1);
+                    } else {
+                        r[e] = 0.0f;   // r(-1)
+                    }
+                }
+                team_sync<G>(team);
+                // the sum over the other edges of every check
+                for (int i = u; i < g.M; i += G) {
+                    const int e0 = __ldg(g.h_ptr + i), d = __ldg(g.h_ptr + i + 1) - e0;
+                    float gk[RM], pre[RM];
+                    float sum = 0.0f;
 #pragma unroll
-                    for (int m = 0; m < kWbpMaxCol; ++m) {
-                        ee[m] = m < d ? __ldg(g.c_edge + c0 + m) : 0;
-                        rr[m] = m < d ? rt[ee[m]] : 0.0f;
-                        pre[m + 1] = pre[m] + rr[m];
+                    for (int k = 0; k < RM; ++k) {
+                        gk[k] = k < d ? x[e0 + k] : 0.0f;
+                        pre[k] = sum;
+                        sum += gk[k];
                     }
                     float suf = 0.0f;
 #pragma unroll
-                    for (int m = kWbpMaxCol - 1; m >= 0; --m) {
-                        ab[m] = 0.0f;
-                        if (m < d && next) {
-                            const float av = lam + (pre[m] + suf);
-                            const float w = __ldg(wv1 + ee[m]);
-                            const bool in = fabsf(w * av) <= clip;
-                            const float qb = QB[ee[m]];
-                            ab[m] = in ? qb * w : 0.0f;
-                            part[(size_t)(T + t + 1) * E + ee[m]] = in ? qb * av : 0.0f;
-                        }
-                        if (m < d) suf += rr[m];
-                    }
-                    float apre[kWbpMaxCol + 1];
-                    apre[0] = 0.0f;
-#pragma unroll
-                    for (int m = 0; m < kWbpMaxCol; ++m) apre[m + 1] = apre[m] + ab[m];
-                    float asuf = 0.0f;
-#pragma unroll
-                    for (int m = kWbpMaxCol - 1; m >= 0; --m) {
-                        if (m < d) {
-                            RB[ee[m]] = gl + (apre[m] + asuf);
-                            asuf += ab[m];
-                        }
+                    for (int k = RM - 1; k >= 0; --k) {
+                        if (k < d) x[e0 + k] = pre[k] + suf;
+                        suf += gk[k];
                     }
                 }
-                __syncwarp();
-                // (2) the check update of iteration t: wc gradient and adjoint of q(t)
-                const float *wc = a.W + (size_t)t * E;
-                for (int i = lane; i < g.M; i += 32) {
-                    const int e0 = __ldg(g.h_ptr + i), d = __ldg(g.h_ptr + i + 1) - e0;
-                    float f[kWbpMaxRow], suf[kWbpMaxRow + 1], gk[kWbpMaxRow];
-                    uint32_t negs = 0, par = syn_bit(sy, i);
-#pragma unroll
-                    for (int k = 0; k < kWbpMaxRow; ++k) {
-                        f[k] = 0.0f;
-                        if (k < d) {
-                            const float x = qt[e0 + k];
-                            f[k] = wphi(fmaxf(fabsf(x), kQmin));
-                            const uint32_t ng = x < 0.0f ? 1u : 0u;
-                            negs |= ng << k;
-                            par ^= ng;
-                        }
-                    }
-                    suf[kWbpMaxRow] = 0.0f;
-#pragma unroll
-                    for (int k = kWbpMaxRow - 1; k >= 0; --k) suf[k] = suf[k + 1] + f[k];
-                    float pre = 0.0f;
-#pragma unroll
-                    for (int k = 0; k < kWbpMaxRow; ++k) {
-                        gk[k] = 0.0f;
-                        if (k < d) {
-                            const float S = pre + suf[k + 1];
-                            const float s = ((par ^ (negs >> k)) & 1u) ? -1.0f : 1.0f;
-                            const float rb = RB[e0 + k];
-                            part[(size_t)t * E + e0 + k] = rb * s * wphi(S);
-                            gk[k] = rb * __ldg(wc + e0 + k) * s * inv_sinh(S);
-                            pre += f[k];
-                        }
-                    }
-                    float gpre[kWbpMaxRow + 1];
-                    gpre[0] = 0.0f;
-#pragma unroll
-                    for (int k = 0; k < kWbpMaxRow; ++k) gpre[k + 1] = gpre[k] + gk[k];
-                    float gsuf = 0.0f;
-#pragma unroll
-                    for (int k = kWbpMaxRow - 1; k >= 0; --k) {
-                        if (k < d) {
-                            const float x = qt[e0 + k];
-                            const float ax = fabsf(x);
-                            const float dq = ax >= kQmin ? (x < 0.0f ? -inv_sinh(ax) : inv_sinh(ax)) : 0.0f;
-                            QB[e0 + k] = dq * (gpre[k] + gsuf);
-                            gsuf += gk[k];
-                        }
-                    }
+                // lambda + the other r(t-1) of every edge
+                var_phase<G, CM>(g, r, u, a.cm, true, [&](int j) { return __ldg(g.lam_col + j); },
+                                 [](int, float, const float (&)[CM]) {});
+                team_sync<G>(team);
+                const float *wv = a.W + (size_t)(T + t) * E;
+                for (int e = u; e < E; e += G) {
+                    const float av = r[e], w = __ldg(wv + e);
+                    const float q = fminf(fmaxf(w * av, -clip), clip), ax = fabsf(q);
+                    const float is = inv_sinh(ax);
+                    const float dq = ax >= kQmin ? (q < 0.0f ? -is : is) : 0.0f;
+                    const float qb = dq * x[e];
+                    const bool in = fabsf(w * av) <= clip;
+                    x[e] = in ? qb * w : 0.0f;
+                    r[e] = in ? qb * av : 0.0f;
                 }
-                __syncwarp();
+            }
+            __syncthreads();
+            // the block's sums over its shots, in shot order
+            for (int n = threadIdx.x; n < 2 * E; n += blockDim.x) {
+                const bool second = n >= E;
+                const int e = second ? n - E : n;
+                const float *src = sm + (second ? E : 3 * E) + e;
+                const size_t at = (size_t)((second ? T : 0) + t) * E + e;
+                Sum2 s;
+                if (base != (int64_t)blockIdx.x * W) {
+                    s.hi = part[at];
+                    s.lo = part[nw + at];
+                }
+                for (int w = 0; w < shots; ++w) s.add(src[(size_t)w * 4 * E]);
+                if (direct) {
+                    grad_w[at] = s.value();
+                } else {
+                    part[at] = s.hi;
+                    part[nw + at] = s.lo;
+                }
             }
         }
-        // q(0) = clip(wv[0] lambda): gradient of wv[0]
-        for (int j = lane; j < g.N; j += 32) {
-            const int c0 = __ldg(g.c_ptr + j), c1 = __ldg(g.c_ptr + j + 1);
-            const float lam = __ldg(g.lam_col + j);
-            for (int c = c0; c < c1; ++c) {
-                const int e = __ldg(g.c_edge + c);
-                const float w = __ldg(a.W + (size_t)T * E + e);
-                part[(size_t)T * E + e] = fabsf(w * lam) <= clip ? QB[e] * lam : 0.0f;
-            }
-        }
-        __syncwarp();
+        __syncthreads();
     }
 }
 
-// out[w] = sum over shots b of part[b][w], in shot order, accumulated in FP64
-__global__ void wbp_reduce_kernel(const float *part, int64_t B, int64_t n, float *out)
+// Sum of the blocks' partial sums in block order: 32 weights x 8 runs of blocks.
+__global__ void __launch_bounds__(256) wbp_reduce_kernel(const float *part, int blocks, int64_t nw, float *out)
 {
-    for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n; w += (int64_t)gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int64_t b = 0; b < B; ++b) s += (double)part[b * n + w];
-        out[w] = (float)s;
+    __shared__ float hi[8][32], lo[8][32];
+    const int lane = threadIdx.x & 31, run = threadIdx.x >> 5;
+    const int64_t w = (int64_t)blockIdx.x * 32 + lane;
+    const int per = (blocks + 7) / 8, b1 = min(blocks, (run + 1) * per);
+    Sum2 s;
+    if (w < nw)
+        for (int b = run * per; b < b1; ++b) {
+            s.add(part[(size_t)b * 2 * nw + w]);
+            s.lo += part[((size_t)b * 2 + 1) * nw + w];
+        }
+    hi[run][lane] = s.hi;
+    lo[run][lane] = s.lo;
+    __syncthreads();
+    if (run == 0 && w < nw) {
+        for (int k = 1; k < 8; ++k) {
+            s.add(hi[k][lane]);
+            s.lo += lo[k][lane];
+        }
+        out[w] = s.value();
     }
+}
+
+
+// Threads per shot: 64 where that gives every SM 16 warps (of the shots an SM gets
+// and has memory for in the adjoint), else 256.  BB[[144,12,12]], T = 20, forward /
+// backward call: 2000 shots 236 / 328 us with 64 threads, 293 / 349 with 256; 1023
+// shots 195 / 237 against 182 / 186; 300 shots 168 / 214 against 124 / 169.
+// Phenomenological BB[[72,12,6]] (1944 edges, 7 shots fit an SM), 3000 shots, T = 6:
+// 438 / 1134 against 360 / 615.
+int team_size(int64_t B, int E)
+{
+    const int64_t per_sm = std::min<int64_t>((B + 151) / 152, (int64_t)(kMaxWbpSmem / ((size_t)16 * E)));
+    return per_sm * 2 >= 16 ? 64 : 256;
+}
+
+// Shots of a block (at most `most`) for an even load: the SM with the most blocks
+// gets as few shots as possible, then the most shots a block.  4096 shots take 4
+// blocks of 7 on an SM instead of 4 of 8 (adjoint 586 -> 502 us with it).  More than
+// 4 blocks do not fit an SM: the teams' named barriers take all 16 of a block, and
+// an SM has 64 (blocks of 3 shots, 27 on an SM, ran 12 at a time: forward 406 us
+// against 328).
+int shots_per_block(int64_t B, int least, int most)
+{
+    int best = most;
+    int64_t load = INT64_MAX;
+    for (int w = most; w >= least; --w) {
+        const int64_t n = ((B + w - 1) / w + 151) / 152;
+        if (n > 4 && w < most) break;
+        if (n * w < load) { best = w; load = n * w; }
+    }
+    return best;
+}
+
+// Shots of a backward block and number of blocks.  Their partial sums (2 x 2 x T x E
+// floats a block) lie before the saved S in the workspace, which leaves at least
+// B (T + 1) E floats: at least four shots a block, and blocks take several rounds of
+// shots where that is short.
+void backward_plan(int64_t B, int E, int T, int G, int *shots, int64_t *blocks)
+{
+    const int most = (int)std::min<size_t>(std::min(8, 1024 / G), kMaxWbpSmem / ((size_t)16 * E));
+    const int64_t room = std::max<int64_t>(1, B * (T + 1) / ((int64_t)4 * T));
+    int w = shots_per_block(B, std::min(4, most), most);
+    while (w < most && (B + w - 1) / w > room) ++w;
+    *shots = (int)std::min<int64_t>(w, B);
+    *blocks = std::min((B + *shots - 1) / *shots, room);
+}
+
+template <typename K>
+cudaError_t allow_smem(K kernel, size_t smem)
+{
+    if (smem <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
 }  // namespace
 
-size_t wbp_smem_forward(int E, int warps) { return (size_t)warps * 2 * E * sizeof(float); }
 size_t wbp_smem_backward(int E, int k, int warps) { return (size_t)warps * (2 * k + 2) * E * sizeof(float); }
 
 cudaError_t launch_wbp_forward(const DevGraph &g, const WbpArgs &a, cudaStream_t s)
 {
     if (a.B <= 0) return cudaSuccess;
-    const int warps = 8;
-    const size_t smem = wbp_smem_forward(a.E, warps);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute((const void *)wbp_forward_kernel,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (a.E > kWbpMaxEdges) return cudaErrorInvalidValue;
+    const int G = team_size(a.B, a.E);
+    const int w = shots_per_block(a.B, 1, std::min(8, 1024 / G));
+    const size_t smem = (size_t)w * a.E * sizeof(float);
+    const int grid = (int)std::min<int64_t>((a.B + w - 1) / w, 152 * 32);
+    auto go = [&](auto kernel) {
+        const cudaError_t e = allow_smem(kernel, smem);
         if (e != cudaSuccess) return e;
-    }
-    const int64_t blocks = (a.B + warps - 1) / warps;
-    const int grid = (int)(blocks < 152 * 32 ? blocks : 152 * 32);
-    wbp_forward_kernel<<<grid, warps * 32, smem, s>>>(g, a);
-    return cudaGetLastError();
+        kernel<<<grid, w * G, smem, s>>>(g, a);
+        return cudaGetLastError();
+    };
+    const bool small = a.cm <= 4 && a.rm <= 8;
+    if (G == 64) return small ? go(wbp_forward_kernel<64, 4, 8>) : go(wbp_forward_kernel<64, kWbpMaxCol, kWbpMaxRow>);
+    return small ? go(wbp_forward_kernel<256, 4, 8>) : go(wbp_forward_kernel<256, kWbpMaxCol, kWbpMaxRow>);
 }
 
 cudaError_t launch_wbp_backward(const DevGraph &g, const WbpArgs &a, float *grad_w, cudaStream_t s)
 {
     const int64_t n = (int64_t)2 * a.T * a.E;
-    if (a.B > 0) {
-        int warps = 4;
-        while (warps > 1 && wbp_smem_backward(a.E, a.k, warps) > kMaxWbpSmem) warps /= 2;
-        const size_t smem = wbp_smem_backward(a.E, a.k, warps);
-        cudaError_t e = cudaFuncSetAttribute((const void *)wbp_backward_kernel,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (a.B <= 0) return cudaMemsetAsync(grad_w, 0, sizeof(float) * n, s);
+    if (a.E > kWbpMaxEdges) return cudaErrorInvalidValue;
+    const int G = team_size(a.B, a.E);
+    int w;
+    int64_t blocks;
+    backward_plan(a.B, a.E, a.T, G, &w, &blocks);
+    const size_t smem = (size_t)w * 4 * a.E * sizeof(float);
+    auto go = [&](auto kernel) {
+        const cudaError_t e = allow_smem(kernel, smem);
         if (e != cudaSuccess) return e;
-        const int64_t blocks = (a.B + warps - 1) / warps;
-        const int grid = (int)(blocks < 152 * 32 ? blocks : 152 * 32);
-        wbp_backward_kernel<<<grid, warps * 32, smem, s>>>(g, a);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        const int rgrid = (int)((n + 255) / 256);
-        wbp_reduce_kernel<<<rgrid, 256, 0, s>>>(a.part, a.B, n, grad_w);
+        kernel<<<(int)blocks, w * G, smem, s>>>(g, a, grad_w);
         return cudaGetLastError();
-    }
-    return cudaMemsetAsync(grad_w, 0, sizeof(float) * n, s);
+    };
+    const bool small = a.cm <= 4 && a.rm <= 8;
+    const cudaError_t e =
+        G == 64 ? (small ? go(wbp_backward_kernel<64, 4, 8>) : go(wbp_backward_kernel<64, kWbpMaxCol, kWbpMaxRow>))
+                : (small ? go(wbp_backward_kernel<256, 4, 8>) : go(wbp_backward_kernel<256, kWbpMaxCol, kWbpMaxRow>));
+    if (e != cudaSuccess || w >= a.B) return e;   // one block in one round has written the gradient
+    wbp_reduce_kernel<<<(int)((n + 31) / 32), 256, 0, s>>>(a.part, (int)blocks, n, grad_w);
+    return cudaGetLastError();
 }
 
 }  // namespace bpdc

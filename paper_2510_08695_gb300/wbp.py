@@ -4,8 +4,8 @@
 over the library's forward kernel (``bpdc_wbp_forward``) and hand-written
 adjoint (``bpdc_decode_backward``): posterior LLRs [B, T, N] of T unrolled
 product-sum iterations with per-edge, per-iteration weights [2, T, E]
-(definition in include/bpdc.h).  Messages are checkpointed every
-``ckpt_every`` iterations and recomputed per segment in the backward pass.
+(definition in include/bpdc.h).  The forward saves what the adjoint needs in
+a workspace whose size depends on ``ckpt_every``; results do not.
 
 ``train_weights`` fits the weights on shots the library samples itself, with
 the binary cross-entropy of the posteriors against the sampled errors, or
