@@ -279,13 +279,16 @@ bool pack(const bpdc_graph_s &g, const Variant &v, Packed &P)
         for (int h = 0; h < 2 * g.w_T; ++h)
             for (size_t a = 0; a < E; ++a) P.wts[(size_t)h * P.slots + edge_slot[a]] = g.w_host[h * E + a];
     }
-    P.chk_idx.assign((size_t)P.pc * P.dc * G, kNoEdge);
+    const bool quad = quad_rows(G, v.dc_max, v.rule);
+    P.chk_idx.assign(quad ? (size_t)std::max(1, (M + 7) / 8) * 32 : (size_t)P.pc * P.dc * G, kNoEdge);
     const int tail_e = v.tail > 0 ? (v.dc_max + v.tail - 1) / v.tail : 0;   // edges per lane in it
     for (int i = 0; i < M; ++i) {
         const int p = i / G, u = i % G;
         for (int a = g.H.ptr[i]; a < g.H.ptr[i + 1]; ++a) {
             const int r = lay.edge_round[a];
-            if (tail && p == P.pc - 1)   // edge r of the pass's u-th check: lane u*tail + r/E, entry r%E
+            if (quad)
+                P.chk_idx[(size_t)(i / 8) * 32 + (i % 8) * 4 + r] = (uint16_t)edge_slot[a];
+            else if (tail && p == P.pc - 1)   // edge r of the pass's u-th check: lane u*tail + r/E, entry r%E
                 P.chk_idx[((size_t)p * P.dc + r % tail_e) * G + u * v.tail + r / tail_e] = (uint16_t)edge_slot[a];
             else
                 P.chk_idx[((size_t)p * P.dc + r) * G + u] = (uint16_t)edge_slot[a];
@@ -294,7 +297,7 @@ bool pack(const bpdc_graph_s &g, const Variant &v, Packed &P)
     // the same edges as word indices of the group's region (12 misc words
     // first; 2 = the +inf word), with the variant's full row width per pass
     // so that a kernel reads every entry of its compile-time width in bounds
-    {
+    if (!quad) {
         const int dcw = std::max(v.dc_max, P.dc);
         P.chk_word.assign((size_t)P.pc * dcw * G, (uint16_t)2);
         for (int p = 0; p < P.pc; ++p)

@@ -38,6 +38,9 @@ constexpr int prof_off(uint64_t prof, int cv, int p)
 // scales them when it loads or stores.  slots_per_lane: the variant's slots of
 // all passes of one lane.
 constexpr bool wide_slots(int G, int slots_per_lane) { return (long)G * slots_per_lane * 4 > 60 * 1024; }
+// Product-sum rows of up to four edges with a warp per shot: four lanes a check
+// (lane 4c + k of round r holds edge k of check 8r + c), chk_idx as [rounds][32].
+constexpr bool quad_rows(int G, int dc_max, int rule) { return G == 32 && dc_max == 4 && rule == 1; }
 // Check-edge word indices per 16-byte entry of the shared-memory edge table.
 constexpr int kTabEdges = 8;
 
@@ -72,7 +75,8 @@ struct DevGraph {
     const float *wts;            // [2][w_T][slots] or null
     int32_t w_T;
     float w_clip;
-    const uint16_t *chk_idx;     // [pc][dc][G] message slot of the check's k-th edge, or kNoEdge
+    const uint16_t *chk_idx;     // [pc][dc][G] message slot of the check's k-th edge, or kNoEdge (quad_rows:
+                                 // [ceil(M/8)][32])
     const uint16_t *chk_word;    // [pc][variant row width][G] the same as word indices of the group's
                                  // region (the +inf word, 2, for none and for padding): read per
                                  // access by the wide kernels

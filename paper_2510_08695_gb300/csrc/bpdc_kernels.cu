@@ -274,7 +274,7 @@ __device__ __forceinline__ void sts32_if(uint32_t a, uint32_t v, bool pred)
 // switches to a batch of another graph).  CMIN: every variable has at least
 // CMIN edges (slots below CMIN need no store predicate); RC: every check has
 // exactly DCM edges.
-template <int G, int PCM, int DCM, int PVM, int CVM, int CMIN, bool RC, uint64_t PROF, bool TAB>
+template <int G, int PCM, int DCM, int PVM, int CVM, int CMIN, bool RC, int RULE, uint64_t PROF, bool TAB>
 struct Lane {
     // slots of pass p (per lane) and the slots before it
     static constexpr int cv(int p) { return prof_cv(PROF, CVM, p); }
@@ -306,8 +306,11 @@ struct Lane {
     // thread) keeps none: it reads the word index of the edge from the
     // read-only table chk_word at each access (coalesced 2-byte loads), so
     // that its registers do not spill.
+    // Four lanes a check (quad_rows): none either, one per round comes from
+    // chk_idx.
+    static constexpr bool kQuad = quad_rows(G, DCM, RULE);
     static constexpr bool kFullAddr = !kWide && PCM * DCM <= 40;
-    static constexpr int kAddrWords = kWide ? 1 : kFullAddr ? PCM * DCM : (PCM * DCM + 1) / 2;
+    static constexpr int kAddrWords = kWide || kQuad ? 1 : kFullAddr ? PCM * DCM : (PCM * DCM + 1) / 2;
     uint32_t aw[kAddrWords];
     const uint16_t *cw;        // wide form: this lane's column of chk_word ([pc][DCM][G])
     uint32_t tab;              // wide form with a table: shared byte address of this lane's entry 0
@@ -396,7 +399,7 @@ struct Lane {
 #pragma unroll
         for (int p = 0; p < PCM; ++p) {
             if (p < g.pc && p * G + u < g.M) cvalid |= 1u << p;
-            if constexpr (!kWide) {
+            if constexpr (!kWide && !kQuad) {
 #pragma unroll
                 for (int k = 0; k < DCM; ++k) {
                     uint32_t v = kNoEdge;
@@ -441,7 +444,7 @@ struct Lane {
 template <int G, int PCM, int DCM, int PVM, int CVM, int CMIN, bool RC, int RULE, uint64_t PROF, bool TAB,
           int TAIL>
 struct Decoder {
-    using L = Lane<G, PCM, DCM, PVM, CVM, CMIN, RC, PROF, TAB>;
+    using L = Lane<G, PCM, DCM, PVM, CVM, CMIN, RC, RULE, PROF, TAB>;
     static constexpr uint32_t kSlot = 4u * G;         // bytes between a variable's slots
     static_assert(TAIL == 0 || (G == 32 && RULE == 0 && (TAIL & (TAIL - 1)) == 0 && TAIL <= 32),
                   "a shared last check pass needs one warp per shot, min-sum and a power-of-two lane count");
@@ -499,6 +502,87 @@ struct Decoder {
             }
         }
         return S;
+    }
+
+    // The product-sum check phase with four lanes a check (quad_rows): round r
+    // holds checks 8r .. 8r+7, lane 4c+k edge k of the c-th (the +inf word where
+    // the check has fewer).  Bound by the instructions of phi (some 60 each): a
+    // lane evaluates two per edge instead of a lane per check evaluating all of
+    // its row's one after the other, the lanes are filled whatever the number of
+    // checks, and the rolled loop over rounds fits the instruction cache, which
+    // up to 13 phi in line for each of four passes did not (no_instruction was
+    // the first stall).  Sums over the other edges keep the order of the edges:
+    // with f1, f2, f3 the values of the lanes at distance 1, 2, 3, prefix plus
+    // suffix is (f2 + f3) + f1 on every lane.  Distance-7 surface code, p = 0.05,
+    // 10^5 shots: 4.24 -> 2.83 ms (issue 65 -> 88 %); distance 9, 2*10^4 shots:
+    // 3.55 -> 2.19 ms.
+    // Returns the row parities (bit 0: unsatisfied) over the rounds.
+    static __device__ __forceinline__ uint32_t quad_checks(const DevGraph &g, const L &ln, int u, int t,
+                                                           uint32_t sbits, bool scatter)
+    {
+        constexpr unsigned kAll = 0xFFFFFFFFu;
+        const int rounds = (g.M + 7) >> 3;
+        const uint16_t *tab = g.chk_idx + u;
+        auto slot = [&](int r) {
+#ifdef BPDC_CHECKS
+            if (!check_index(3, (long long)r * 32 + u, g.n_chk_idx)) return (uint32_t)kNoEdge;
+#endif
+            return (uint32_t)__ldg(tab + r * 32);
+        };
+        uint32_t unsat = 0;
+        uint32_t v = rounds > 0 ? slot(0) : kNoEdge;
+#pragma unroll 1
+        for (int r = 0; r < rounds; ++r) {
+            const bool own = v != kNoEdge;
+            const uint32_t a = own ? ln.slot_base + 4u * v : ln.inf_addr;
+            if (r + 1 < rounds) v = slot(r + 1);
+            const float q = ldsf(a);
+            const float av = fabsf(q);
+            uint32_t S = __float_as_uint(q) ^ ((sbits >> r) & 1u) * 0x80000001u;
+            S ^= __shfl_xor_sync(kAll, S, 1);
+            S ^= __shfl_xor_sync(kAll, S, 2);
+            unsat |= S;
+            if (!scatter) continue;
+            const float o = __shfl_xor_sync(kAll, av, 1);
+            const float lo = fminf(av, o), hi = fmaxf(av, o);
+            const float lo2 = __shfl_xor_sync(kAll, lo, 2), hi2 = __shfl_xor_sync(kAll, hi, 2);
+            const float mn1 = fminf(lo, lo2), mid = fmaxf(lo, lo2), mid2 = fminf(hi, hi2);
+            const float mn2 = fminf(mid, mid2), mn3 = fmaxf(mid, mid2);
+            // a check with at most two finite inputs sends each the other one
+            // unchanged; else phi of the sum of the others' phi, with the
+            // arguments lowered by sa, or by sb on a single minimum edge, whose
+            // own sum starts at min2 (see phi)
+            const bool pair = mn3 == f_inf(), is_min = av == mn1;
+            const float sa = fminf(fmaxf(mn1 - kPhiShift, 0.0f), kLlrCap);
+            const float sb = fminf(fmaxf(mn2 - kPhiShift, 0.0f), kLlrCap);
+            const float f = phi(av - sa);
+            const float f1 = __shfl_xor_sync(kAll, f, 1), f2 = __shfl_xor_sync(kAll, f, 2), f3 = __shfl_xor_sync(kAll, f, 3);
+            float arg = (f2 + f3) + f1, shift = sa;
+            if (__any_sync(kAll, sb != sa)) {
+                const float w = is_min ? 0.0f : phi(av - sb);
+                const float w1 = __shfl_xor_sync(kAll, w, 1), w2 = __shfl_xor_sync(kAll, w, 2), w3 = __shfl_xor_sync(kAll, w, 3);
+                // the sum in the order of the edges, without this lane's own
+                const int k = u & 3;
+                const float x = k < 2 ? w1 : w2, y = k == 0 ? w2 : w3, z = k == 0 ? w3 : k == 1 ? w2 : w1;
+                if (sb != sa && is_min) {
+                    arg = (x + y) + z;
+                    shift = sb;
+                }
+            }
+            float mag = shift + phi(arg);
+            if (pair) mag = scaled_min(1.0f, is_min ? mn2 : mn1);
+            mag = fminf(mag, kLlrCap);
+            uint32_t out = __float_as_uint(mag) ^ (S & 0x80000000u) ^ (__float_as_uint(q) & 0x80000000u);
+            if (g.wts && own) {   // weighted BP: r *= wc
+                const size_t at = (size_t)(min(t, g.w_T) - 1) * g.slots + ((a - ln.slot_base) >> 2);
+#ifdef BPDC_CHECKS
+                check_index(8, (long long)at, g.n_wts);
+#endif
+                out = __float_as_uint(__ldg(g.wts + at) * __uint_as_float(out));
+            }
+            if (own) sts32(a, out);
+        }
+        return unsat;
     }
 
     // Initial messages of a BP run: every variable announces its prior LLR
@@ -619,8 +703,9 @@ struct Decoder {
             const bool scatter = t <= T;
             uint32_t unsat = 0;
             // ---- check phase ----
+            if constexpr (L::kQuad) unsat = quad_checks(g, ln, u, t, sbits, scatter);
 #pragma unroll
-            for (int p = 0; p < PCM; ++p) {
+            for (int p = 0; p < (L::kQuad ? 0 : PCM); ++p) {
                 if constexpr (TAIL > 0) {
                     if (p == PCM - 1) {   // every lane takes part in the shared last pass
                         if (FAST || p < g.pc) unsat |= tail_pass(ln, p, sbits, alpha, scatter);
@@ -979,8 +1064,12 @@ struct Decoder {
             // ---- a1: syndrome bits of my checks ----
             uint32_t sbits = 0;
             const uint32_t *sy = bd.syn + (size_t)b * g.MW;
+            if constexpr (L::kQuad) {   // bit r on the first lane of each check of round r
+                for (int i = u >> 2, r = 0; i < g.M; i += 8, ++r)
+                    if ((u & 3) == 0) sbits |= ((__ldg(sy + (i >> 5)) >> (i & 31)) & 1u) << r;
+            }
 #pragma unroll
-            for (int p = 0; p < PCM; ++p) {
+            for (int p = 0; p < (L::kQuad ? 0 : PCM); ++p) {
                 // a shared last pass: the first lane of each check holds its bit
                 const bool tail = TAIL > 0 && p == PCM - 1;
                 const int i = tail ? p * G + u / (TAIL > 0 ? TAIL : 1) : p * G + u;
@@ -1021,7 +1110,7 @@ struct Decoder {
                         grp.sync();
                     }
                     int iters = 0;
-                    const bool ok = (g.pc == PCM && g.pv == PVM && !post_row)
+                    const bool ok = ((L::kQuad || g.pc == PCM) && g.pv == PVM && !post_row)
                                         ? run<true>(g, ln, grp, sbits, hd, iters, post_row)
                                         : run<false>(g, ln, grp, sbits, hd, iters, post_row);
                     if (second) it2 = iters; else it1 = iters;
