@@ -258,7 +258,7 @@ int bpdc_decode_host(const bpdc_batch *batches, int32_t n_batches, int64_t chunk
  * process exits.  The caller still passes every input and output, and the
  * graphs must already exist.
  *   - At most 16 batches per call, all on graphs that use the same kernel
- *     variant (bpdc_graph_info.kernel_id), and at most 2^32 - 2^24 shots in
+ *     variant (bpdc_graph_info.kernel_id; 20 and 21 count as one), and at most 2^32 - 2^24 shots in
  *     all; otherwise BPDC_ERR_UNSUPPORTED with a message, and nothing is
  *     launched.
  *   - The first call on a device looks up the array's device address; make

@@ -382,7 +382,7 @@ int plan_and_upload(bpdc_graph_s *g, int want_G, int want_id = -1)
     // before the plain form of the same shape), then the 256- and 512-thread
     // groups (a slot-profile variant before the uniform one of the same shape:
     // it is faster wherever its profile fits the graph)
-    static const int kOrder[] = {19, 17, 20, 7, 0, 12, 5, 11, 15, 1, 3, 2, 4, 6, 16, 14, 13, 18};
+    static const int kOrder[] = {19, 17, 21, 20, 7, 0, 12, 5, 11, 15, 1, 3, 2, 4, 6, 16, 14, 13, 18};
     Packed P{};
     int vid = -1;
     for (int id : kOrder) {
@@ -1078,8 +1078,8 @@ int bpdc_decode_multi_noalloc(const bpdc_batch *batches, int32_t n, void *stream
         if (!batches[i].graph) return fail(BPDC_ERR_INVALID_ARG, "batch %d has no graph", i);
         if (batches[i].graph->device != dev) return fail(BPDC_ERR_INVALID_ARG, "graphs on different devices");
         if (batches[i].B < 0) return fail(BPDC_ERR_INVALID_ARG, "batch %d: B < 0", i);
-        if (vid < 0) vid = batches[i].graph->variant;
-        if (batches[i].graph->variant != vid)
+        if (vid < 0) vid = variant_family(batches[i].graph->variant);
+        if (variant_family(batches[i].graph->variant) != vid)
             return fail(BPDC_ERR_UNSUPPORTED, "bpdc_decode_multi_noalloc needs every graph on one kernel variant");
         if (batches[i].B == 0) continue;
         if (!batches[i].syndromes) return fail(BPDC_ERR_INVALID_ARG, "batch %d: syndromes NULL", i);
@@ -1090,29 +1090,38 @@ int bpdc_decode_multi_noalloc(const bpdc_batch *batches, int32_t n, void *stream
     std::lock_guard<std::mutex> lk(owner->mu);
     DeviceGuard dgd(dev);
     if (!dgd.ok) return fail(BPDC_ERR_CUDA, "cannot select device %d", dev);
-    BatchDesc descs[kStaticBatches];   // host stack: no allocation
-    int cnt = 0, smem = 0, bps = 0;
-    int64_t total = 0;
-    for (int i = 0; i < n; ++i) {
-        const bpdc_batch &bt = batches[i];
-        if (bt.B == 0) continue;
-        fill_desc(descs[cnt], bt.graph, bt.B, bt.syndromes, bt.shot_offset, &bt.out, total);
-        total += bt.B;
-        if (bt.graph->smem_bytes >= smem) {
-            smem = bt.graph->smem_bytes;
-            bps = bt.graph->blocks_per_sm;
-        }
-        ++cnt;
-    }
-    if (cnt == 0) return BPDC_OK;
-    if (total > kMaxLaunchShots)
+    int64_t all = 0;
+    for (int i = 0; i < n; ++i) all += batches[i].B;
+    if (all > kMaxLaunchShots)
         return fail(BPDC_ERR_UNSUPPORTED, "at most %lld shots per call (got %lld)", (long long)kMaxLaunchShots,
-                    (long long)total);
-    const Variant &v = variant(vid);
-    const int64_t need = (total + v.block_threads / v.G - 1) / (v.block_threads / v.G);
-    const int64_t grid = std::min<int64_t>((int64_t)owner->sm_count * bps, need);
-    cudaError_t e = launch_variant_static(vid, descs, cnt, total, (int)grid, smem, (cudaStream_t)stream);
-    return e == cudaSuccess ? BPDC_OK : cuda_fail(e, "allocation-free decode launch");
+                    (long long)all);
+    // one launch per variant of the family, in the order of the first batch of each
+    bool done[kStaticBatches] = {};
+    for (int k = 0; k < n; ++k) {
+        if (done[k] || batches[k].B == 0) continue;
+        const int id = batches[k].graph->variant;
+        BatchDesc descs[kStaticBatches];   // host stack: no allocation
+        int cnt = 0, smem = 0, bps = 0;
+        int64_t total = 0;
+        for (int i = k; i < n; ++i) {
+            const bpdc_batch &bt = batches[i];
+            if (bt.B == 0 || bt.graph->variant != id) continue;
+            done[i] = true;
+            fill_desc(descs[cnt], bt.graph, bt.B, bt.syndromes, bt.shot_offset, &bt.out, total);
+            total += bt.B;
+            if (bt.graph->smem_bytes >= smem) {
+                smem = bt.graph->smem_bytes;
+                bps = bt.graph->blocks_per_sm;
+            }
+            ++cnt;
+        }
+        const Variant &v = variant(id);
+        const int64_t need = (total + v.block_threads / v.G - 1) / (v.block_threads / v.G);
+        const int64_t grid = std::min<int64_t>((int64_t)owner->sm_count * bps, need);
+        cudaError_t e = launch_variant_static(id, descs, cnt, total, (int)grid, smem, (cudaStream_t)stream);
+        if (e != cudaSuccess) return cuda_fail(e, "allocation-free decode launch");
+    }
+    return BPDC_OK;
 }
 
 int bpdc_cut_select(bpdc_graph_t g, int64_t B, const float *posterior_llr, uint64_t shot_offset,

@@ -146,6 +146,7 @@ struct Variant {
     uint64_t prof;       // slots per variable pass (prof_cv); 0: cv_max in every pass
     bool tab;            // check-edge table in shared memory (wide form only)
     int tail;            // lanes per check of a shared last check pass (0: none; one warp per shot)
+    int np, nv;          // check and variable passes loaded together
 };
 
 // Placement of variables on positions and order of the edges inside each
@@ -163,6 +164,9 @@ void plan_layout(int M, int N, const std::vector<int32_t> &row_ptr, const std::v
                  int npos, int dc, bool optimize, const std::vector<int> &pass_cv, Layout &out);
 
 int num_variants();
+// Variants whose graphs an allocation-free launch may mix: one and its
+// specialisation to a smaller shape (variant 21 takes graphs that 20 takes too).
+constexpr int variant_family(int id) { return id == 21 ? 20 : id; }
 // Checked builds: the first failed bounds check since the last call (site 0:
 // none) and its index, then cleared.  Normal builds return false.
 bool check_status(int *site, long long *index);

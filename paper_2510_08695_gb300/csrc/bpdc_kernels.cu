@@ -238,6 +238,72 @@ __device__ __forceinline__ float fmin3(float a, float b, float c)
     return r;
 }
 
+// The same of the three magnitudes, and their maximum.
+__device__ __forceinline__ float fmin3_abs(float a, float b, float c)
+{
+    float r;
+    asm("min.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float fmax3_abs(float a, float b, float c)
+{
+    float r;
+    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// The two smallest magnitudes and the XOR of the words of a row, taken three, two
+// or one edges at a time.  Of three words a, b, c the least m and the greatest M
+// magnitude take one instruction each, and the middle one is what is left of
+// their XOR (needed anyway, for the parities) without m and M, up to the sign:
+// 7.5 instructions for three edges where pairs take 9 (the ALU pipe is the first
+// bound of the check update).  Exact in any order.  2-5 % of a decode: HGP-2500 p =
+// 0.06, 20000 shots 10.18 -> 9.97 ms; BB[[144,12,12]] p = 0.08, 10^5 shots 1.81 ->
+// 1.76 ms; phenomenological p = 0.006, 10^5 shots 9.02 -> 8.56 ms.
+struct RowMin {
+    float mn1, mn2;
+    uint32_t S;   // bit 31: sign parity, bit 0: hard-decision parity
+    __device__ __forceinline__ explicit RowMin(uint32_t s) : mn1(f_inf()), mn2(f_inf()), S(s) {}
+    __device__ __forceinline__ void merge(float lo, float hi)   // lo >= 0; the sign of hi is ignored
+    {
+        mn2 = fmin3_abs(mn2, fmaxf(mn1, lo), hi);
+        mn1 = fminf(mn1, lo);
+    }
+    __device__ __forceinline__ void take3(float a, float b, float c, bool first)
+    {
+        const uint32_t x = __float_as_uint(a) ^ __float_as_uint(b) ^ __float_as_uint(c);
+        const float m = fmin3_abs(a, b, c), M = fmax3_abs(a, b, c);
+        const float mid = __uint_as_float(x ^ __float_as_uint(m) ^ __float_as_uint(M));
+        S ^= x;
+        if (first) {
+            mn1 = m;
+            mn2 = fabsf(mid);
+        } else {
+            merge(m, mid);
+        }
+    }
+    __device__ __forceinline__ void take2(float a, float b)
+    {
+        S ^= __float_as_uint(a) ^ __float_as_uint(b);
+        merge(fminf(fabsf(a), fabsf(b)), fmaxf(fabsf(a), fabsf(b)));
+    }
+    __device__ __forceinline__ void take1(float a)
+    {
+        S ^= __float_as_uint(a);
+        mn2 = fminf(mn2, fmaxf(mn1, fabsf(a)));
+        mn1 = fminf(mn1, fabsf(a));
+    }
+    template <int D>
+    __device__ __forceinline__ void take_all(const float (&q)[D])
+    {
+        constexpr int kThree = D / 3 * 3;
+#pragma unroll
+        for (int k = 0; k < kThree; k += 3) take3(q[k], q[k + 1], q[k + 2], k == 0);
+        if constexpr (D - kThree == 2) take2(q[D - 2], q[D - 1]);
+        else if constexpr (D - kThree == 1) take1(q[D - 1]);
+    }
+};
+
 // 16-byte load of a table entry (four words).
 __device__ __forceinline__ uint4 lds128(uint32_t a)
 {
@@ -333,8 +399,14 @@ struct Lane {
         return (vm[n >> 5] >> (n & 31)) & 1u;
     }
 
-    // Shared byte address of the word with index w of the group's region.
-    __device__ __forceinline__ uint32_t word_addr(uint32_t w) const { return region_base + 4u * w; }
+    // Shared byte addresses of the words of the group's region whose indices lie
+    // in the low and high half of w: the dot product of the halves with (4, 0) or
+    // (0, 4) extracts, scales and adds in one instruction, off the ALU pipe that
+    // bounds the long rows (a mask or shift and a scaled add took two of its slots
+    // at each of the four accesses of an edge: 2000 circuit-level BB[[144,12,12]]
+    // shots 26.2 -> 23.3 ms).
+    __device__ __forceinline__ uint32_t low_addr(uint32_t w) const { return __dp2a_lo(w, 0x0004u, region_base); }
+    __device__ __forceinline__ uint32_t high_addr(uint32_t w) const { return __dp2a_lo(w, 0x0400u, region_base); }
 
     __device__ __forceinline__ uint32_t addr(int p, int k) const
     {
@@ -346,7 +418,7 @@ struct Lane {
         } else {
             const int n = p * DCM + k;
             if constexpr (kFullAddr) return aw[n];
-            else return (n & 1) ? (aw[n >> 1] >> 16) : (aw[n >> 1] & 0xFFFFu);
+            else return __dp2a_lo(aw[n >> 1], (n & 1) ? 0x0100u : 0x0001u, 0u);
         }
     }
 
@@ -440,9 +512,11 @@ struct Lane {
 };
 
 // TAIL > 0 (one warp per shot): the last check pass holds up to 32 / TAIL
-// checks, each spread over TAIL consecutive lanes (see tail_pass).
+// checks, each spread over TAIL consecutive lanes (see tail_pass).  NP, NV: check
+// and variable passes whose loads are all issued before the first of them is
+// reduced and stored (more registers, less waiting).
 template <int G, int PCM, int DCM, int PVM, int CVM, int CMIN, bool RC, int RULE, uint64_t PROF, bool TAB,
-          int TAIL>
+          int TAIL, int NP, int NV>
 struct Decoder {
     using L = Lane<G, PCM, DCM, PVM, CVM, CMIN, RC, RULE, PROF, TAB>;
     static constexpr uint32_t kSlot = 4u * G;         // bytes between a variable's slots
@@ -628,60 +702,120 @@ struct Decoder {
     // the extrinsic messages q = lambda + the other r (prefix and suffix
     // sums), stored tagged with e; at the last iteration slot 0 keeps the
     // tagged L for the cut selection.  Slots past a variable's degree hold 0,
-    // so a pass wider than the degree adds exact zeros.  Returns e.
-    template <bool FAST, int P>
-    static __device__ __forceinline__ uint32_t var_pass(const DevGraph &g, const L &ln, int u, int t, bool last,
-                                                        float *post_row)
+    // so a pass wider than the degree adds exact zeros.  Returns e in every bit.
+    template <bool FAST, int P, int N>
+    static __device__ __forceinline__ uint32_t var_group(const DevGraph &g, const L &ln, int u, int t, bool last,
+                                                         float *post_row)
     {
-        constexpr int CVP = L::cv(P);
-        const uint32_t base = pass_base(ln, P);
-        float r[CVP];
+        float r[N][CVM];
+        uint32_t hd = 0;
 #pragma unroll
-        for (int m = 0; m < CVP; ++m) r[m] = __uint_as_float(lds32(base + m * kSlot));
-        float pre[CVP + 1];
-        pre[0] = ln.lamv[P];
+        for (int i = 0; i < N; ++i)
 #pragma unroll
-        for (int m = 0; m < CVP; ++m) pre[m + 1] = pre[m] + r[m];
-        float suf[CVP + 1];
-        suf[CVP] = 0.0f;
-        suf[CVP - 1] = r[CVP - 1];
+            for (int m = 0; m < CVM; ++m)
+                if (m < L::cv(P + i)) r[i][m] = __uint_as_float(lds32(pass_base(ln, P + i) + m * kSlot));
 #pragma unroll
-        for (int m = CVP - 2; m >= 1; --m) suf[m] = r[m] + suf[m + 1];
-        const float Lp = pre[CVP];
-        const uint32_t e = Lp <= 0.0f ? 1u : 0u;
-        const float *wv = (RULE == 1 && g.wts)
-            ? g.wts + ((size_t)g.w_T + min(t + 1, g.w_T) - 1) * g.slots + L::off(P) * G + u
-            : nullptr;
+        for (int i = 0; i < N; ++i) {
+            const int p = P + i, cvp = L::cv(p);
+            const uint32_t base = pass_base(ln, p);
+            float pre[CVM + 1], suf[CVM + 1];
+            pre[0] = ln.lamv[p];
 #pragma unroll
-        for (int m = 0; m < CVP; ++m) {
-            float q = (m == CVP - 1) ? pre[m] : pre[m] + suf[m + 1];
-            if (RULE == 1 && wv) q = fminf(fmaxf(__ldg(wv + m * G) * q, -g.w_clip), g.w_clip);
-            const uint32_t qv = (__float_as_uint(q) & ~1u) | e;
-            if (m < CMIN) sts32(base + m * kSlot, qv);
-            else sts32_if(base + m * kSlot, qv, ln.has(P, m));
-        }
-        if (last) {   // slot 0 keeps L for the cut selection
-            const uint32_t lv = (__float_as_uint(Lp) & ~1u) | e;
-            if (CMIN > 0) sts32(base, lv);
-            else sts32_if(base, lv, ln.has(P, 0));
-        }
+            for (int m = 0; m < CVM; ++m)
+                if (m < cvp) pre[m + 1] = pre[m] + r[i][m];
+#pragma unroll
+            for (int m = CVM - 1; m >= 1; --m)
+                if (m < cvp) suf[m] = m == cvp - 1 ? r[i][m] : r[i][m] + suf[m + 1];
+            const float Lp = pre[cvp];
+            const uint32_t e = Lp <= 0.0f ? 1u : 0u;
+            hd |= e << p;
+            const float *wv = (RULE == 1 && g.wts)
+                ? g.wts + ((size_t)g.w_T + min(t + 1, g.w_T) - 1) * g.slots + L::off(p) * G + u
+                : nullptr;
+#pragma unroll
+            for (int m = 0; m < CVM; ++m) {
+                if (m >= cvp) continue;
+                float q = (m == cvp - 1) ? pre[m] : pre[m] + suf[m + 1];
+                if (RULE == 1 && wv) q = fminf(fmaxf(__ldg(wv + m * G) * q, -g.w_clip), g.w_clip);
+                const uint32_t qv = (__float_as_uint(q) & ~1u) | e;
+                if (m < CMIN) sts32(base + m * kSlot, qv);
+                else sts32_if(base + m * kSlot, qv, ln.has(p, m));
+            }
+            if (last) {   // slot 0 keeps L for the cut selection
+                const uint32_t lv = (__float_as_uint(Lp) & ~1u) | e;
+                if (CMIN > 0) sts32(base, lv);
+                else sts32_if(base, lv, ln.has(p, 0));
+            }
 #ifdef BPDC_CHECKS
-        if (!FAST && post_row && ((ln.vvalid >> P) & 1u) && !post_ok(g, (long long)P * G + u)) {} else
+            if (!FAST && post_row && ((ln.vvalid >> p) & 1u) && !post_ok(g, (long long)p * G + u)) {} else
 #endif
-        if (!FAST && post_row && ((ln.vvalid >> P) & 1u)) post_row[__ldg(g.pos_col + P * G + u)] = Lp;
-        return e;
+            if (!FAST && post_row && ((ln.vvalid >> p) & 1u)) post_row[__ldg(g.pos_col + p * G + u)] = Lp;
+        }
+        return hd;
     }
 
     // The variable updates of passes P .. PVM-1 (all passes of the variant on
-    // the fast path, else those the graph occupies); ORs decision bit p of
-    // each pass into nhd.
+    // the fast path, NV at a time, else those the graph occupies); ORs decision
+    // bit p of each pass into nhd.
     template <bool FAST, int P>
     static __device__ __forceinline__ void var_passes(const DevGraph &g, const L &ln, int u, int t, bool last,
                                                       float *post_row, uint32_t &nhd)
     {
         if constexpr (P < PVM) {
-            if (FAST || P < g.pv) nhd |= var_pass<FAST, P>(g, ln, u, t, last, post_row) << P;
-            var_passes<FAST, P + 1>(g, ln, u, t, last, post_row, nhd);
+            constexpr int N = !FAST ? 1 : (PVM - P < NV) ? (PVM - P) : NV;
+            if (FAST || P < g.pv) nhd |= var_group<FAST, P, N>(g, ln, u, t, last, post_row);
+            var_passes<FAST, P + N>(g, ln, u, t, last, post_row, nhd);
+        }
+    }
+
+    // Min-sum check updates of passes P .. P+N-1 with the rows held in registers,
+    // for a lane that has a check in each: every row is gathered before the
+    // first is reduced and scattered, so that their latencies overlap.
+    template <int P, int N>
+    static __device__ __forceinline__ void held_rows(const L &ln, uint32_t sbits, float alpha, bool scatter,
+                                                     uint32_t &unsat)
+    {
+        float q[N][DCM];
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+#pragma unroll
+            for (int k = 0; k < DCM; ++k) q[i][k] = ldsf(ln.addr(P + i, k));
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            RowMin row(((sbits >> (P + i)) & 1u) * 0x80000001u);
+            row.template take_all<DCM>(q[i]);
+            unsat |= row.S;
+            if (scatter) {
+                const float sa = __uint_as_float(__float_as_uint(alpha) ^ (row.S & 0x80000000u));
+                const uint32_t m1 = __float_as_uint(scaled_min(sa, row.mn1));
+                const uint32_t m2 = __float_as_uint(scaled_min(sa, row.mn2));
+#pragma unroll
+                for (int k = 0; k < DCM; ++k) {
+                    const uint32_t a = ln.addr(P + i, k);
+                    const uint32_t out = (fabsf(q[i][k]) == row.mn1 ? m2 : m1) ^ (__float_as_uint(q[i][k]) & 0x80000000u);
+                    if (RC) sts32(a, out);
+                    else sts32_if(a, out, a != ln.inf_addr);
+                }
+            }
+        }
+    }
+
+    // The check passes P .. END-1 of the fast path, NP at a time; lanes without a
+    // check in the variant's last pass skip it.
+    template <int P, int END>
+    static __device__ __forceinline__ void held_passes(const L &ln, uint32_t sbits, float alpha, bool scatter,
+                                                       uint32_t &unsat)
+    {
+        if constexpr (P < END) {
+            constexpr int N = (END - P < NP) ? (END - P) : NP;
+            if constexpr (P + N < PCM) {
+                held_rows<P, N>(ln, sbits, alpha, scatter, unsat);
+            } else if ((ln.cvalid >> (PCM - 1)) & 1u) {
+                held_rows<P, N>(ln, sbits, alpha, scatter, unsat);
+            } else if constexpr (N > 1) {
+                held_rows<P, N - 1>(ln, sbits, alpha, scatter, unsat);
+            }
+            held_passes<P + N, END>(ln, sbits, alpha, scatter, unsat);
         }
     }
 
@@ -703,9 +837,14 @@ struct Decoder {
             const bool scatter = t <= T;
             uint32_t unsat = 0;
             // ---- check phase ----
+            constexpr bool kGroup = FAST && RULE == 0 && DCM <= 16 && (NP > 1);
             if constexpr (L::kQuad) unsat = quad_checks(g, ln, u, t, sbits, scatter);
+            if constexpr (kGroup) {
+                held_passes<0, (TAIL > 0 ? PCM - 1 : PCM)>(ln, sbits, alpha, scatter, unsat);
+                if constexpr (TAIL > 0) unsat |= tail_pass(ln, PCM - 1, sbits, alpha, scatter);
+            }
 #pragma unroll
-            for (int p = 0; p < (L::kQuad ? 0 : PCM); ++p) {
+            for (int p = 0; p < (L::kQuad || kGroup ? 0 : PCM); ++p) {
                 if constexpr (TAIL > 0) {
                     if (p == PCM - 1) {   // every lane takes part in the shared last pass
                         if (FAST || p < g.pc) unsat |= tail_pass(ln, p, sbits, alpha, scatter);
@@ -728,102 +867,77 @@ struct Decoder {
                     uint32_t S = ((sbits >> p) & 1u) * 0x80000001u;
                     if constexpr (RULE == 0) {
                         // normalized min-sum
-                        float mn1 = f_inf(), mn2 = f_inf();
+                        RowMin row(S);
                         float qf[kHold ? DCM : 1];
                         float qh[L::kHoldLong ? DCM : 1];   // q of a long row (table form)
-                        auto gather = [&](int k) {
-                            // unused slots point at the group's +inf word
-                            const float v = ldsf(ln.addr(p, k));
-                            if constexpr (kHold) qf[k] = v;
-                            S ^= __float_as_uint(v);   // bit 31: sign parity, bit 0: hard-decision parity
-                            const float av = fabsf(v);
-                            mn2 = fminf(mn2, fmaxf(mn1, av));
-                            mn1 = fminf(mn1, av);
-                        };
                         if constexpr (kHold) {
-                            // edges in pairs: with lo <= hi the pair's
-                            // smallest two, the second minimum of the four
-                            // values {mn1 <= mn2, lo, hi} is
-                            // min(mn2, max(mn1, lo), hi)
-                            auto gather2 = [&](int k, bool first) {
-                                const float va = ldsf(ln.addr(p, k)), vb = ldsf(ln.addr(p, k + 1));
-                                qf[k] = va;
-                                qf[k + 1] = vb;
-                                S ^= __float_as_uint(va) ^ __float_as_uint(vb);
-                                const float lo = fminf(fabsf(va), fabsf(vb)), hi = fmaxf(fabsf(va), fabsf(vb));
-                                if (first) {
-                                    mn1 = lo;
-                                    mn2 = hi;
-                                } else {
-                                    mn2 = fmin3(mn2, fmaxf(mn1, lo), hi);
-                                    mn1 = fminf(mn1, lo);
-                                }
-                            };
+                            // unused slots point at the group's +inf word
 #pragma unroll
-                            for (int k = 0; k + 1 < DCM; k += 2) gather2(k, k == 0);
-                            if (DCM & 1) gather(DCM - 1);
+                            for (int k = 0; k < DCM; ++k) qf[k] = ldsf(ln.addr(p, k));
+                            row.take_all(qf);
                         } else if constexpr (L::kTab) {
                             // the lane's edge word indices come from its shared
-                            // table, 8 per 16-byte load; the two edges of a word
-                            // go through the pairwise minimum (mn1 = mn2 = +inf
-                            // before the first pair gives the first pair's
-                            // order statistics)
-                            auto take = [&](float va, float vb) {
-                                S ^= __float_as_uint(va) ^ __float_as_uint(vb);
-                                const float lo = fminf(fabsf(va), fabsf(vb)), hi = fmaxf(fabsf(va), fabsf(vb));
-                                mn2 = fmin3(mn2, fmaxf(mn1, lo), hi);
-                                mn1 = fminf(mn1, lo);
-                            };
-                            auto take1 = [&](float v) {
-                                S ^= __float_as_uint(v);
-                                const float av = fabsf(v);
-                                mn2 = fminf(mn2, fmaxf(mn1, av));
-                                mn1 = fminf(mn1, av);
-                            };
+                            // table, 8 per 16-byte load
                             constexpr int kFull = DCM / kTabEdges, kTail = DCM % kTabEdges;
                             if constexpr (L::kHoldLong) {
                                 // every chunk unrolled, the q of the row kept in qh
+                                uint32_t ww[L::kTabChunks * 4] = {};
+                                auto get = [&](int k) {
+                                    const uint32_t w = ww[k >> 1];
+                                    return qh[k] = ldsf((k & 1) ? ln.high_addr(w) : ln.low_addr(w));
+                                };
 #pragma unroll
                                 for (int c = 0; c < L::kTabChunks; ++c) {
                                     const uint4 w = lds128(ln.tab_entry(p, c));
-                                    const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+                                    ww[4 * c] = w.x;
+                                    ww[4 * c + 1] = w.y;
+                                    ww[4 * c + 2] = w.z;
+                                    ww[4 * c + 3] = w.w;
+                                    // the triples whose last edge lies in this chunk
 #pragma unroll
-                                    for (int h = 0; h < 4; ++h) {
-                                        const int k = c * kTabEdges + 2 * h;
-                                        if (k + 1 < DCM) {
-                                            qh[k] = ldsf(ln.word_addr(ww[h] & 0xFFFFu));
-                                            qh[k + 1] = ldsf(ln.word_addr(ww[h] >> 16));
-                                            take(qh[k], qh[k + 1]);
-                                        } else if (k < DCM) {
-                                            qh[k] = ldsf(ln.word_addr(ww[h] & 0xFFFFu));
-                                            take1(qh[k]);
+                                    for (int k = 0; k + 2 < DCM; k += 3)
+                                        if ((k + 2) / kTabEdges == c) {
+                                            const float a0 = get(k), a1 = get(k + 1), a2 = get(k + 2);
+                                            row.take3(a0, a1, a2, k == 0);
                                         }
-                                    }
+                                }
+                                constexpr int kThree = DCM / 3 * 3;
+                                if constexpr (DCM - kThree == 2) {
+                                    const float a0 = get(kThree), a1 = get(kThree + 1);
+                                    row.take2(a0, a1);
+                                } else if constexpr (DCM - kThree == 1) {
+                                    row.take1(get(kThree));
                                 }
                             } else {
-                                auto pair = [&](uint32_t w) {
-                                    take(ldsf(ln.word_addr(w & 0xFFFFu)), ldsf(ln.word_addr(w >> 16)));
-                                };
+                                auto lo = [&](uint32_t w) { return ldsf(ln.low_addr(w)); };
+                                auto hi = [&](uint32_t w) { return ldsf(ln.high_addr(w)); };
 #pragma unroll 1
                                 for (int c = 0; c < kFull; ++c) {
                                     const uint4 w = lds128(ln.tab_entry(p, c));
-                                    pair(w.x);
-                                    pair(w.y);
-                                    pair(w.z);
-                                    pair(w.w);
+                                    const float a0 = lo(w.x), a1 = hi(w.x), a2 = lo(w.y), a3 = hi(w.y);
+                                    row.take3(a0, a1, a2, false);
+                                    const float a4 = lo(w.z), a5 = hi(w.z);
+                                    row.take3(a3, a4, a5, false);
+                                    const float a6 = lo(w.w), a7 = hi(w.w);
+                                    row.take2(a6, a7);
                                 }
                                 if constexpr (kTail > 0) {
                                     const uint4 w = lds128(ln.tab_entry(p, kFull));
                                     const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-                                    for (int h = 0; h < kTail / 2; ++h) pair(ww[h]);
-                                    if constexpr (kTail & 1) take1(ldsf(ln.word_addr(ww[kTail / 2] & 0xFFFFu)));
+                                    for (int h = 0; h < kTail / 2; ++h) {
+                                        const float a0 = lo(ww[h]), a1 = hi(ww[h]);
+                                        row.take2(a0, a1);
+                                    }
+                                    if constexpr (kTail & 1) row.take1(lo(ww[kTail / 2]));
                                 }
                             }
                         } else {   // long rows: bounded unrolling keeps few loads in flight
 #pragma unroll 5
-                            for (int k = 0; k < DCM; ++k) gather(k);
+                            for (int k = 0; k < DCM; ++k) row.take1(ldsf(ln.addr(p, k)));
                         }
+                        S = row.S;
+                        const float mn1 = row.mn1, mn2 = row.mn2;
                         unsat |= S;
                         if (scatter) {
                             // the minimum over the other edges is min2 for the edge
@@ -866,16 +980,16 @@ struct Decoder {
 #pragma unroll
                                         for (int h = 0; h < 4; ++h) {
                                             const int k = c * kTabEdges + 2 * h;
-                                            if (k < DCM) store(ln.word_addr(ww[h] & 0xFFFFu), out_of(qh[k]));
-                                            if (k + 1 < DCM) store(ln.word_addr(ww[h] >> 16), out_of(qh[k + 1]));
+                                            if (k < DCM) store(ln.low_addr(ww[h]), out_of(qh[k]));
+                                            if (k + 1 < DCM) store(ln.high_addr(ww[h]), out_of(qh[k + 1]));
                                         }
                                     }
                                 } else {
                                     // each q read again from its slot, then overwritten by r
                                     auto put_at = [&](uint32_t a) { store(a, out_of(ldsf(a))); };
                                     auto put2 = [&](uint32_t w) {
-                                        put_at(ln.word_addr(w & 0xFFFFu));
-                                        put_at(ln.word_addr(w >> 16));
+                                        put_at(ln.low_addr(w));
+                                        put_at(ln.high_addr(w));
                                     };
 #pragma unroll 1
                                     for (int c = 0; c < kFull; ++c) {
@@ -890,7 +1004,7 @@ struct Decoder {
                                         const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
                                         for (int h = 0; h < kTail / 2; ++h) put2(ww[h]);
-                                        if constexpr (kTail & 1) put_at(ln.word_addr(ww[kTail / 2] & 0xFFFFu));
+                                        if constexpr (kTail & 1) put_at(ln.low_addr(ww[kTail / 2]));
                                     }
                                 }
                             } else {
@@ -1212,14 +1326,14 @@ struct Decoder {
 };
 
 template <int G, int PCM, int DCM, int PVM, int CVM, int CMIN, bool RC, int RULE, int BLOCK, int MINB,
-          uint64_t PROF, bool TAB, int TAIL>
+          uint64_t PROF, bool TAB, int TAIL, int NP, int NV>
 __global__ void __launch_bounds__(BLOCK, MINB) decode_kernel(LaunchDesc ld, int region_words)
 {
     extern __shared__ uint32_t smem[];
     const int tid = threadIdx.x;
-    const int gib = tid / G;
+    const int gib = G == BLOCK ? 0 : tid / G;   // one group: its addresses are constants
     Group<G> grp;
-    grp.u = tid % G;
+    grp.u = G == BLOCK ? tid : tid % G;
     grp.bar = 1 + gib;
     if constexpr (G <= 32) {
         const int wl = tid & 31;
@@ -1231,7 +1345,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) decode_kernel(LaunchDesc ld, int 
         grp.leader = 0;
     }
     uint32_t *region = smem + (size_t)gib * region_words;
-    Decoder<G, PCM, DCM, PVM, CVM, CMIN, RC, RULE, PROF, TAB, TAIL>::decode(ld, region, grp, gib);
+    Decoder<G, PCM, DCM, PVM, CVM, CMIN, RC, RULE, PROF, TAB, TAIL, NP, NV>::decode(ld, region, grp, gib);
 }
 
 // Cut selection alone, one block per shot (same selection code as the fused kernel).
@@ -1264,7 +1378,8 @@ __global__ void cut_select_kernel(DevGraph g, int64_t B, const float *post, uint
 // weight, minimum column weight, regular rows, check rule (0 min-sum,
 // 1 product-sum), block threads, min blocks per SM, slots per variable pass
 // (3 bits per pass, 0: the column weight in every pass), shared edge table,
-// lanes per check of a shared last check pass (0: none)).
+// lanes per check of a shared last check pass (0: none), check passes and variable
+// passes loaded together).
 // Variants 13 and 14 take circuit-level detector models (rows of up to 35
 // edges, one shot per SM): 13 with 6 slots in every pass and the check-edge
 // indices read from global memory at each access, 14 with variables sorted by
@@ -1279,33 +1394,40 @@ __global__ void cut_select_kernel(DevGraph g, int64_t B, const float *post, uint
 // and three variable passes of a warp: its fast path) at 4 and 6 blocks per SM.
 // Variants 19 and 20 are variants 17 and 7 with the last check pass shared
 // (BB[[72,12,6]]: its 4 checks past the first 32 on 8 lanes each;
-// BB[[144,12,12]]: its 8 checks past the first 64 on 4 lanes each).
+// BB[[144,12,12]]: its 8 checks past the first 64 on 4 lanes each).  Variant 21 has
+// the shape of BB[[108,8,10]] (two check and four variable passes, which took the
+// guarded path of a three- and five-pass variant: 2*10^5 shots at p = 0.04 771 ->
+// 566 us).  The last two numbers are the check and variable passes whose loads
+// are issued together: more than one pays where a warp has registers left and a
+// shot's latency counts (variant 20: 64 shots of BB[[144,12,12]] 74 -> 65 us, 2*10^5
+// 724 -> 713 us; HGP-2500 and BB[[72,12,6]] gained nothing).
 #define BPDC_VARIANTS(X)                                                       \
-    X(0, 32, 3, 6, 5, 3, 3, true, 0, 256, 4, 0, false, 0)                      \
-    X(1, 256, 5, 7, 10, 4, 3, true, 0, 256, 3, 0, false, 0)                    \
-    X(2, 512, 3, 7, 5, 4, 3, true, 0, 512, 2, 0, false, 0)                     \
-    X(3, 256, 4, 8, 11, 3, 2, false, 0, 256, 3, 0, false, 0)                   \
-    X(4, 512, 2, 8, 6, 3, 2, false, 0, 512, 2, 0, false, 0)                    \
-    X(5, 32, 4, 8, 8, 4, 1, false, 0, 256, 4, 0, false, 0)                     \
-    X(6, 128, 10, 7, 20, 4, 3, true, 0, 128, 6, 0, false, 0)                   \
-    X(7, 32, 3, 6, 5, 3, 3, true, 0, 256, 3, 0, false, 0)                      \
-    X(8, 256, 5, 7, 10, 4, 3, true, 0, 256, 2, 0, false, 0)                    \
-    X(9, 512, 3, 7, 5, 4, 3, true, 0, 512, 1, 0, false, 0)                     \
-    X(10, 256, 4, 8, 11, 3, 2, false, 0, 256, 2, 0, false, 0)                  \
-    X(11, 32, 4, 4, 4, 2, 1, false, 1, 256, 4, 0, false, 0)                    \
-    X(12, 32, 3, 6, 5, 3, 3, true, 1, 256, 4, 0, false, 0)                     \
-    X(13, 1024, 1, 35, 9, 6, 2, false, 0, 1024, 1, 0, false, 0)                \
-    X(14, 1024, 1, 35, 9, 6, 2, false, 0, 1024, 1, 0x36db72eull, true, 0)      \
-    X(15, 256, 5, 7, 10, 4, 3, true, 0, 256, 3, 0x1b6db924ull, false, 0)       \
-    X(16, 512, 2, 35, 18, 6, 2, false, 0, 512, 1, 0x136db6db6e4b76ull, true, 0) \
-    X(17, 32, 2, 6, 3, 3, 3, true, 0, 256, 4, 0, false, 0)                     \
-    X(18, 32, 2, 6, 3, 3, 3, true, 0, 256, 6, 0, false, 0)                     \
-    X(19, 32, 2, 6, 3, 3, 3, true, 0, 256, 4, 0, false, 8)                     \
-    X(20, 32, 3, 6, 5, 3, 3, true, 0, 256, 3, 0, false, 4)
+    X(0, 32, 3, 6, 5, 3, 3, true, 0, 256, 4, 0, false, 0, 1, 1)                \
+    X(1, 256, 5, 7, 10, 4, 3, true, 0, 256, 3, 0, false, 0, 1, 1)              \
+    X(2, 512, 3, 7, 5, 4, 3, true, 0, 512, 2, 0, false, 0, 1, 1)               \
+    X(3, 256, 4, 8, 11, 3, 2, false, 0, 256, 3, 0, false, 0, 1, 1)             \
+    X(4, 512, 2, 8, 6, 3, 2, false, 0, 512, 2, 0, false, 0, 1, 1)              \
+    X(5, 32, 4, 8, 8, 4, 1, false, 0, 256, 4, 0, false, 0, 1, 1)               \
+    X(6, 128, 10, 7, 20, 4, 3, true, 0, 128, 6, 0, false, 0, 1, 1)             \
+    X(7, 32, 3, 6, 5, 3, 3, true, 0, 256, 3, 0, false, 0, 1, 1)                \
+    X(8, 256, 5, 7, 10, 4, 3, true, 0, 256, 2, 0, false, 0, 1, 1)              \
+    X(9, 512, 3, 7, 5, 4, 3, true, 0, 512, 1, 0, false, 0, 1, 1)               \
+    X(10, 256, 4, 8, 11, 3, 2, false, 0, 256, 2, 0, false, 0, 1, 1)            \
+    X(11, 32, 4, 4, 4, 2, 1, false, 1, 256, 4, 0, false, 0, 1, 1)              \
+    X(12, 32, 3, 6, 5, 3, 3, true, 1, 256, 4, 0, false, 0, 1, 1)               \
+    X(13, 1024, 1, 35, 9, 6, 2, false, 0, 1024, 1, 0, false, 0, 1, 1)          \
+    X(14, 1024, 1, 35, 9, 6, 2, false, 0, 1024, 1, 0x36db72eull, true, 0, 1, 1) \
+    X(15, 256, 5, 7, 10, 4, 3, true, 0, 256, 3, 0x1b6db924ull, false, 0, 1, 1) \
+    X(16, 512, 2, 35, 18, 6, 2, false, 0, 512, 1, 0x136db6db6e4b76ull, true, 0, 1, 1) \
+    X(17, 32, 2, 6, 3, 3, 3, true, 0, 256, 4, 0, false, 0, 1, 1)               \
+    X(18, 32, 2, 6, 3, 3, 3, true, 0, 256, 6, 0, false, 0, 1, 1)               \
+    X(19, 32, 2, 6, 3, 3, 3, true, 0, 256, 4, 0, false, 8, 1, 1)               \
+    X(20, 32, 3, 6, 5, 3, 3, true, 0, 256, 3, 0, false, 4, 2, 5)               \
+    X(21, 32, 2, 6, 4, 3, 3, true, 0, 256, 4, 0, false, 0, 1, 1)              
 
 static const Variant kVariants[] = {
-#define X(id, G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL) \
-    {id, G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL},
+#define X(id, G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV) \
+    {id, G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV},
     BPDC_VARIANTS(X)
 #undef X
 };
@@ -1331,8 +1453,8 @@ bool check_status(int *, long long *) { return false; }
 static const void *variant_fn(int id)
 {
     switch (id) {
-#define X(id, G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL) \
-    case id: return (const void *)decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL>;
+#define X(id, G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV) \
+    case id: return (const void *)decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV>;
         BPDC_VARIANTS(X)
 #undef X
     default: return nullptr;
@@ -1381,9 +1503,9 @@ cudaError_t launch_variant(int id, const LaunchDesc &ld, int grid, int smem_byte
 {
     const int region = smem_bytes / 4 / (kVariants[id].block_threads / kVariants[id].G);
     switch (id) {
-#define X(id, G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL)                          \
+#define X(id, G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV)                          \
     case id:                                                                                        \
-        decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL>                  \
+        decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV>                  \
             <<<grid, BLK, smem_bytes, s>>>(ld, region);                                             \
         return cudaGetLastError();
         BPDC_VARIANTS(X)
