@@ -253,7 +253,7 @@ int bpdc_decode_host(const bpdc_batch *batches, int32_t n_batches, int64_t chunk
  * allocator, code embedded in a host framework whose allocator owns all device
  * memory, or a stream that is being captured into a CUDA graph.  This call
  * allocates nothing: the persistent kernel's scratch (its device work counter
- * and the descriptors of up to 16 batches: 256 + 16 x 344 = 5760 bytes) lives in a fixed device
+ * and the descriptors of up to 16 batches: 256 + 16 x 368 = 6144 bytes) lives in a fixed device
  * array of the library, which every GPU that loads the library holds until the
  * process exits.  The caller still passes every input and output, and the
  * graphs must already exist.
@@ -263,15 +263,16 @@ int bpdc_decode_host(const bpdc_batch *batches, int32_t n_batches, int64_t chunk
  *     launched.
  *   - The first call on a device looks up the array's device address; make
  *     that first call before any stream capture on that device.
- *   - Every call reuses the same array (the work counter is cleared at the
- *     start of each call).  Calls whose launches overlap on the GPU, e.g. on
+ *   - Every call reuses the same array (each decode leaves the work counter at
+ *     zero for the next).  Calls whose launches overlap on the GPU, e.g. on
  *     two streams, race on it: keep such calls ordered on one stream.
- *   - The call issues two kernel launches and nothing else: a setup kernel that
- *     receives the batch descriptors as kernel parameters, writes them into the
- *     array and clears the counter, then the decode kernel.  It can therefore
- *     be captured into a CUDA graph (after a first uncaptured call on the
- *     device); each replay decodes whatever the captured syndrome buffers hold
- *     into the captured output buffers.
+ *   - The call issues kernel launches and nothing else: the decode kernel, which
+ *     carries up to four batch descriptors in its parameters, and for more
+ *     batches a setup kernel before it that receives them as parameters and
+ *     writes them into the array (both once more where variants 20 and 21 are
+ *     mixed).  It can therefore be captured into a CUDA graph (after a first
+ *     uncaptured call on the device); each replay decodes whatever the captured
+ *     syndrome buffers hold into the captured output buffers.
  * Results equal those of bpdc_decode_multi on the same batches. */
 int bpdc_decode_multi_noalloc(const bpdc_batch *batches, int32_t n_batches, void *stream);
 

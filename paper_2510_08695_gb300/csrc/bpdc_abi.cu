@@ -526,6 +526,10 @@ int ring_init(bpdc_graph_s *g)
         e = cudaEventCreateWithFlags(&g->ring[s].done, cudaEventDisableTiming);
         if (e != cudaSuccess) return cuda_fail(e, "event creation");
     }
+    // every launch leaves its work counter at 0 for the next one on its slot
+    e = cudaMemset2D(g->ring_mem, per, 0, sizeof(unsigned long long), kRing);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
+    if (e != cudaSuccess) return cuda_fail(e, "work counters");
     return BPDC_OK;
 }
 
@@ -575,41 +579,36 @@ void fill_desc(BatchDesc &d, const bpdc_graph_s *g, int64_t B, const uint32_t *s
     d.cut_in = o->cut_in;
 }
 
-// Enqueues one launch of variant `vid` over n descriptors (already filled in
-// the host mirror of ring slot s).
-int enqueue(bpdc_graph_s *g, int s, int n, int64_t total, int vid, int smem, bool persistent,
-            cudaStream_t stream)
+// Descriptors of a launch on ring slot rs: up to kInlineBatches travel with the
+// launch (ld), more in the slot's pinned mirror.
+BatchDesc *desc_of(LaunchDesc &ld, const RingSlot &rs, int k) { return k < kInlineBatches ? &ld.own[k] : &rs.host_desc[k]; }
+
+// Enqueues one launch of variant `vid` over the n descriptors written by desc_of
+// on ring slot s; smem, bps: shared memory and residency of its widest graph.  The
+// only work on the stream besides the kernel is a copy of the descriptors where
+// there are more than a launch's parameters hold (a request of 64 BB[[72,12,6]]
+// shots, call after call: 46 -> 38 us with the blocks of launch_shape).
+int enqueue(bpdc_graph_s *g, int s, LaunchDesc &ld, int n, int64_t total, int vid, int smem, int bps,
+            bool persistent, cudaStream_t stream)
 {
     if (total > kMaxLaunchShots)
         return fail(BPDC_ERR_UNSUPPORTED, "at most %lld shots per launch (got %lld)", (long long)kMaxLaunchShots,
                     (long long)total);
     RingSlot &rs = g->ring[s];
-    cudaError_t e = cudaMemcpyAsync(rs.dev_desc, rs.host_desc, sizeof(BatchDesc) * n,
-                                    cudaMemcpyHostToDevice, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "descriptor upload");
-    LaunchDesc ld{};
-    ld.batches = rs.dev_desc;
+    cudaError_t e;
+    ld.batches = nullptr;
+    if (n > kInlineBatches) {
+        for (int k = 0; k < kInlineBatches; ++k) rs.host_desc[k] = ld.own[k];
+        e = cudaMemcpyAsync(rs.dev_desc, rs.host_desc, sizeof(BatchDesc) * n, cudaMemcpyHostToDevice, stream);
+        if (e != cudaSuccess) return cuda_fail(e, "descriptor upload");
+        ld.batches = rs.dev_desc;
+    }
     ld.n_batches = n;
     ld.total = total;
-    ld.work = nullptr;
-    const Variant &v = variant(vid);
-    const int gpb = v.block_threads / v.G;
-    int bps = 0, regs = 0;
-    e = variant_attributes(vid, smem, &bps, &regs);
-    if (e != cudaSuccess) return cuda_fail(e, "kernel attributes");
-    if (bps < 1) return fail(BPDC_ERR_UNSUPPORTED, "kernel variant %d not resident with %d bytes", vid, smem);
-    int64_t grid;
-    const int64_t need = (total + gpb - 1) / gpb;
-    if (persistent) {
-        e = cudaMemsetAsync(rs.work, 0, sizeof(unsigned long long), stream);
-        if (e != cudaSuccess) return cuda_fail(e, "work counter reset");
-        ld.work = (unsigned int *)rs.work;
-        grid = std::min<int64_t>((int64_t)g->sm_count * bps, need);
-    } else {
-        grid = need;
-    }
-    if (grid > 0x7FFFFFFF) return fail(BPDC_ERR_UNSUPPORTED, "batch too large for one launch");
-    e = launch_variant(vid, ld, (int)grid, smem, stream);
+    ld.work = persistent ? rs.work : nullptr;
+    const LaunchShape shape = launch_shape(variant(vid), total, persistent, g->sm_count, bps);
+    if (shape.grid > 0x7FFFFFFF) return fail(BPDC_ERR_UNSUPPORTED, "batch too large for one launch");
+    e = launch_variant(vid, ld, (int)shape.grid, shape.groups, smem, stream);
     if (e != cudaSuccess) return cuda_fail(e, "decode launch");
     e = cudaEventRecord(rs.done, stream);
     if (e != cudaSuccess) return cuda_fail(e, "event record");
@@ -874,8 +873,9 @@ int bpdc_decode(bpdc_graph_t g, int64_t B, const uint32_t *syndromes, uint64_t s
     std::lock_guard<std::mutex> lk(g->mu);
     DeviceGuard dgd(g->device);
     const int s = acquire_slot(g);
-    fill_desc(g->ring[s].host_desc[0], g, B, syndromes, shot_offset, out, 0);
-    return enqueue(g, s, 1, B, g->variant, g->smem_bytes, persistent != 0, (cudaStream_t)stream);
+    LaunchDesc ld{};
+    fill_desc(ld.own[0], g, B, syndromes, shot_offset, out, 0);
+    return enqueue(g, s, ld, 1, B, g->variant, g->smem_bytes, g->blocks_per_sm, persistent != 0, (cudaStream_t)stream);
 }
 
 int bpdc_decode_multi(const bpdc_batch *batches, int32_t n, void *stream)
@@ -905,22 +905,26 @@ int bpdc_decode_multi(const bpdc_batch *batches, int32_t n, void *stream)
     while (i < order.size()) {
         const int vid = batches[order[i]].graph->variant;
         const int s = acquire_slot(owner);
-        int cnt = 0, smem = 0;
+        int cnt = 0, smem = 0, bps = 0;
         int64_t total = 0;
+        LaunchDesc ld{};
         while (i < order.size() && cnt < kMaxBatches && batches[order[i]].graph->variant == vid) {
             const bpdc_batch &bt = batches[order[i]];
             // a launch takes at most kMaxLaunchShots: the next one takes the rest
             if (cnt > 0 && total + bt.B > kMaxLaunchShots) break;
             if (bt.B > 0) {
-                fill_desc(owner->ring[s].host_desc[cnt], bt.graph, bt.B, bt.syndromes, bt.shot_offset, &bt.out, total);
+                fill_desc(*desc_of(ld, owner->ring[s], cnt), bt.graph, bt.B, bt.syndromes, bt.shot_offset, &bt.out, total);
                 total += bt.B;
-                smem = std::max(smem, bt.graph->smem_bytes);
+                if (bt.graph->smem_bytes >= smem) {   // the widest graph bounds the residency
+                    smem = bt.graph->smem_bytes;
+                    bps = bt.graph->blocks_per_sm;
+                }
                 ++cnt;
             }
             ++i;
         }
         if (cnt == 0) continue;
-        int rc = enqueue(owner, s, cnt, total, vid, smem, true, (cudaStream_t)stream);
+        int rc = enqueue(owner, s, ld, cnt, total, vid, smem, bps, true, (cudaStream_t)stream);
         if (rc != BPDC_OK) return rc;
     }
     return BPDC_OK;
@@ -1031,8 +1035,9 @@ int bpdc_decode_host(const bpdc_batch *batches, int32_t n, int64_t chunk_shots, 
             o.obs_true = bt.out.obs_true ? d_obs : nullptr;
             o.iterations = bt.out.iterations ? d_it : nullptr;
             const int slot = acquire_slot(owner);
-            fill_desc(owner->ring[slot].host_desc[0], g, nb, d_syn, bt.shot_offset + (uint64_t)b0, &o, 0);
-            rc = enqueue(owner, slot, 1, nb, g->variant, g->smem_bytes, true, cs);
+            LaunchDesc ld{};
+            fill_desc(ld.own[0], g, nb, d_syn, bt.shot_offset + (uint64_t)b0, &o, 0);
+            rc = enqueue(owner, slot, ld, 1, nb, g->variant, g->smem_bytes, g->blocks_per_sm, true, cs);
             if (rc != BPDC_OK) break;
             e = cudaEventRecord(owner->ev_dec[s], cs);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(owner->copy_out, owner->ev_dec[s], 0);
@@ -1115,10 +1120,8 @@ int bpdc_decode_multi_noalloc(const bpdc_batch *batches, int32_t n, void *stream
             }
             ++cnt;
         }
-        const Variant &v = variant(id);
-        const int64_t need = (total + v.block_threads / v.G - 1) / (v.block_threads / v.G);
-        const int64_t grid = std::min<int64_t>((int64_t)owner->sm_count * bps, need);
-        cudaError_t e = launch_variant_static(id, descs, cnt, total, (int)grid, smem, (cudaStream_t)stream);
+        const LaunchShape shape = launch_shape(variant(id), total, true, owner->sm_count, bps);
+        cudaError_t e = launch_variant_static(id, descs, cnt, total, shape, smem, (cudaStream_t)stream);
         if (e != cudaSuccess) return cuda_fail(e, "allocation-free decode launch");
     }
     return BPDC_OK;

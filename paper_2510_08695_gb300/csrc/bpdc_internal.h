@@ -126,11 +126,17 @@ struct BatchDesc {
     const uint32_t *cut_in;
 };
 
+// Descriptors that a launch carries in its own parameters: a request (one batch)
+// or a few need no copy to the device before the kernel.
+constexpr int kInlineBatches = 4;
+
 struct LaunchDesc {
-    const BatchDesc *batches;    // device array
+    BatchDesc own[kInlineBatches];
+    const BatchDesc *batches;    // device array of more than kInlineBatches, else null: `own`
     int32_t n_batches;
     int64_t total;               // shots over all batches
-    unsigned int *work;          // persistent work counter (nullptr: one group per shot)
+    unsigned long long *work;    // persistent work counter, 0 before the launch and after it (nullptr: one
+                                 // group per shot)
 };
 
 // A compiled kernel variant and its limits.
@@ -173,7 +179,16 @@ bool check_status(int *site, long long *index);
 const Variant &variant(int id);
 // Occupancy query and launch of variant `id`.
 cudaError_t variant_attributes(int id, int smem_bytes, int *blocks_per_sm, int *regs);
-cudaError_t launch_variant(int id, const LaunchDesc &ld, int grid, int smem_bytes, cudaStream_t s);
+// smem_bytes: of a full block (block_threads / G groups); groups: the groups a block of this launch has.
+cudaError_t launch_variant(int id, const LaunchDesc &ld, int grid, int groups, int smem_bytes, cudaStream_t s);
+// Groups per block and blocks of a launch of `total` shots: a persistent one fills
+// the chip with bps full blocks per SM at most; fewer shots than that are spread
+// over the SMs first.
+struct LaunchShape {
+    int groups;
+    int64_t grid;
+};
+LaunchShape launch_shape(const Variant &v, int64_t total, bool persistent, int sm_count, int bps);
 
 // Most shots one decode launch takes: the kernel keeps shot indices and work
 // tickets in 32 bits (groups of more than 32 threads pass the ticket through a
@@ -187,7 +202,7 @@ constexpr int kStaticBatches = 16;
 // Launch of variant `id` whose work counter and batch descriptors live in the
 // library's fixed device scratch array instead of caller- or library-allocated
 // memory.  host_descs: n <= kStaticBatches descriptors in host memory.
-cudaError_t launch_variant_static(int id, const BatchDesc *host_descs, int n, int64_t total, int grid,
+cudaError_t launch_variant_static(int id, const BatchDesc *host_descs, int n, int64_t total, LaunchShape shape,
                                   int smem_bytes, cudaStream_t s);
 
 cudaError_t launch_cut_select(const DevGraph &g, int64_t B, const float *post, uint64_t shot_offset,

@@ -1097,6 +1097,7 @@ struct Decoder {
     static __device__ void decode(const LaunchDesc &ld, uint32_t *region, const Group<G> &grp, int gib)
     {
         const int u = grp.u;
+        const BatchDesc *const batches = ld.batches ? ld.batches : ld.own;
         L ln;
         // little state lives across the iterations (the loop needs the
         // registers): shot indices are 32-bit (a launch holds fewer than 2^32
@@ -1120,8 +1121,16 @@ struct Decoder {
             uint32_t w;
             if (ld.work) {
                 unsigned long long x = 0;
+                // every group draws one ticket past the last shot; the last of
+                // those leaves the counter at 0 for the next launch
+                auto draw = [&]() {
+                    const unsigned long long y = atomicAdd(ld.work, 1ull);
+                    if (y == (unsigned long long)ld.total + (unsigned long long)gridDim.x * groups_per_block - 1ull)
+                        *ld.work = 0ull;
+                    return y;
+                };
                 if constexpr (G <= 32) {
-                    if (u == 0) x = atomicAdd((unsigned long long *)ld.work, 1ull);
+                    if (u == 0) x = draw();
                     x = __shfl_sync(grp.mask, x, grp.leader);
                 } else {
                     // the ticket goes through a shared word (two, alternating);
@@ -1131,7 +1140,7 @@ struct Decoder {
                     // or staging (of another graph, perhaps) before every lane
                     // has copied out the previous shot
                     uint32_t *misc = region + 0;
-                    if (u == 0) misc[bufsel] = (uint32_t)atomicAdd((unsigned long long *)ld.work, 1ull);
+                    if (u == 0) misc[bufsel] = (uint32_t)draw();
                     grp.sync();
                     x = misc[bufsel];
                     bufsel ^= 1u;
@@ -1145,25 +1154,25 @@ struct Decoder {
             if ((int64_t)w >= ld.total) break;
             if (w < bfirst || w >= bend) {
                 if (u == 0) {
-                    if (bi >= 0 && ld.batches[bi].counters)
-                        for (int x = 0; x < 4; ++x) atomicAdd(ld.batches[bi].counters + x, cnt[x]);
+                    if (bi >= 0 && batches[bi].counters)
+                        for (int x = 0; x < 4; ++x) atomicAdd(batches[bi].counters + x, cnt[x]);
                     cnt[0] = cnt[1] = cnt[2] = cnt[3] = 0;
                 }
                 int lo = 0, hi = ld.n_batches - 1;
                 while (lo < hi) {  // last batch with first <= w
                     const int mid = (lo + hi + 1) >> 1;
-                    if (ld.batches[mid].first <= (int64_t)w) lo = mid; else hi = mid - 1;
+                    if (batches[mid].first <= (int64_t)w) lo = mid; else hi = mid - 1;
                 }
-                const DevGraph &gnew = ld.batches[lo].g;
-                if (bi < 0 || gnew.chk_idx != ld.batches[bi].g.chk_idx || gnew.lam != ld.batches[bi].g.lam) {
+                const DevGraph &gnew = batches[lo].g;
+                if (bi < 0 || gnew.chk_idx != batches[bi].g.chk_idx || gnew.lam != batches[bi].g.lam) {
                     ln.load(gnew, u, slot_base, inf_word);
                     lam_dirty = false;
                 }
                 bi = lo;
-                bfirst = (uint32_t)ld.batches[bi].first;
-                bend = bfirst + (uint32_t)ld.batches[bi].B;
+                bfirst = (uint32_t)batches[bi].first;
+                bend = bfirst + (uint32_t)batches[bi].B;
             }
-            const BatchDesc &bd = ld.batches[bi];
+            const BatchDesc &bd = batches[bi];
             // the graph's fields are read where they are used (L1 hits), not
             // copied per shot: a copy of the whole descriptor took registers
             // and stack from the iterations (2-10 % slower)
@@ -1320,14 +1329,14 @@ struct Decoder {
                 cnt[3] += ran_dc ? 1 : 0;
             }
         }
-        if (bi >= 0 && u == 0 && ld.batches[bi].counters)
-            for (int x = 0; x < 4; ++x) atomicAdd(ld.batches[bi].counters + x, cnt[x]);
+        if (bi >= 0 && u == 0 && batches[bi].counters)
+            for (int x = 0; x < 4; ++x) atomicAdd(batches[bi].counters + x, cnt[x]);
     }
 };
 
 template <int G, int PCM, int DCM, int PVM, int CVM, int CMIN, bool RC, int RULE, int BLOCK, int MINB,
           uint64_t PROF, bool TAB, int TAIL, int NP, int NV>
-__global__ void __launch_bounds__(BLOCK, MINB) decode_kernel(LaunchDesc ld, int region_words)
+__global__ void __launch_bounds__(BLOCK, MINB) decode_kernel(const __grid_constant__ LaunchDesc ld, int region_words)
 {
     extern __shared__ uint32_t smem[];
     const int tid = threadIdx.x;
@@ -1499,19 +1508,34 @@ cudaError_t variant_attributes(int id, int smem_bytes, int *blocks_per_sm, int *
     return cudaSuccess;
 }
 
-cudaError_t launch_variant(int id, const LaunchDesc &ld, int grid, int smem_bytes, cudaStream_t s)
+cudaError_t launch_variant(int id, const LaunchDesc &ld, int grid, int groups, int smem_bytes, cudaStream_t s)
 {
     const int region = smem_bytes / 4 / (kVariants[id].block_threads / kVariants[id].G);
+    const int threads = groups * kVariants[id].G, smem = groups * region * 4;
     switch (id) {
 #define X(id, G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV)                          \
     case id:                                                                                        \
         decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV>                  \
-            <<<grid, BLK, smem_bytes, s>>>(ld, region);                                             \
+            <<<grid, threads, smem, s>>>(ld, region);                                               \
         return cudaGetLastError();
         BPDC_VARIANTS(X)
 #undef X
     default: return cudaErrorInvalidValue;
     }
+}
+
+LaunchShape launch_shape(const Variant &v, int64_t total, bool persistent, int sm_count, int bps)
+{
+    const int full = v.block_threads / v.G;
+    // up to a full block's shots per SM: blocks of as many groups as an even
+    // spread over the SMs needs (64 BB[[144,12,12]] shots on 64 SMs instead of 8:
+    // 67 -> 49 us a call together with the launch's own descriptors)
+    const int64_t even = (total + sm_count - 1) / sm_count;
+    LaunchShape s;
+    s.groups = (int)(even < full ? even : full);
+    s.grid = (total + s.groups - 1) / s.groups;
+    if (persistent && s.grid > (int64_t)sm_count * bps) s.grid = (int64_t)sm_count * bps;
+    return s;
 }
 
 // ---------------------------------------------------------------------------
@@ -1555,34 +1579,36 @@ struct StaticSetup {
     int n;
 };
 
-__global__ void static_setup_kernel(StaticSetup st, BatchDesc *dst, unsigned long long *work)
+__global__ void static_setup_kernel(StaticSetup st, BatchDesc *dst)
 {
     const int i = threadIdx.x;
     if (i < st.n) dst[i] = st.d[i];
-    if (i == 0) *work = 0ull;   // the work counter starts at zero
 }
 
-cudaError_t launch_variant_static(int id, const BatchDesc *host_descs, int n, int64_t total, int grid,
+cudaError_t launch_variant_static(int id, const BatchDesc *host_descs, int n, int64_t total, LaunchShape shape,
                                   int smem_bytes, cudaStream_t s)
 {
     if (n < 1 || n > kStaticBatches) return cudaErrorInvalidValue;
     void *base = nullptr;
     cudaError_t e = static_scratch_address(&base);
     if (e != cudaSuccess) return e;
-    auto *work = reinterpret_cast<unsigned long long *>(base);
-    auto *descs = reinterpret_cast<BatchDesc *>(static_cast<unsigned char *>(base) + 256);
-    StaticSetup st;
-    for (int i = 0; i < n; ++i) st.d[i] = host_descs[i];
-    st.n = n;
-    static_setup_kernel<<<1, 32, 0, s>>>(st, descs, work);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
     LaunchDesc ld{};
-    ld.batches = descs;
+    ld.work = reinterpret_cast<unsigned long long *>(base);   // 0 at load time, and again after each launch
     ld.n_batches = n;
     ld.total = total;
-    ld.work = reinterpret_cast<unsigned int *>(work);
-    return launch_variant(id, ld, grid, smem_bytes, s);
+    if (n <= kInlineBatches) {
+        for (int i = 0; i < n; ++i) ld.own[i] = host_descs[i];
+    } else {
+        auto *descs = reinterpret_cast<BatchDesc *>(static_cast<unsigned char *>(base) + 256);
+        StaticSetup st;
+        for (int i = 0; i < n; ++i) st.d[i] = host_descs[i];
+        st.n = n;
+        static_setup_kernel<<<1, 32, 0, s>>>(st, descs);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        ld.batches = descs;
+    }
+    return launch_variant(id, ld, (int)shape.grid, shape.groups, smem_bytes, s);
 }
 
 cudaError_t launch_cut_select(const DevGraph &g, int64_t B, const float *post, uint64_t shot_offset,
