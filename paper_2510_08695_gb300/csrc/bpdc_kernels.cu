@@ -540,17 +540,21 @@ struct Decoder {
     // first lane carries the syndrome bit.  A short last pass (a few checks
     // past a multiple of 32) thus costs about a lane's share of a full one.
     // Returns the check's parity word (bit 0: unsatisfied).
-    static __device__ __forceinline__ uint32_t tail_pass(const L &ln, int p, uint32_t sbits, float alpha,
-                                                         bool scatter)
+    static constexpr int kTailEdges = (DCM + TAIL - 1) / (TAIL > 0 ? TAIL : 1);   // edges per lane
+    static __device__ __forceinline__ void tail_gather(const L &ln, int p, float (&qf)[kTailEdges])
     {
-        constexpr int E = (DCM + TAIL - 1) / (TAIL > 0 ? TAIL : 1);   // edges per lane
+#pragma unroll
+        for (int k = 0; k < kTailEdges; ++k) qf[k] = ldsf(ln.addr(p, k));
+    }
+    static __device__ __forceinline__ uint32_t tail_pass(const L &ln, int p, uint32_t sbits, float alpha,
+                                                         bool scatter, const float (&qf)[kTailEdges])
+    {
+        constexpr int E = kTailEdges;
         uint32_t S = ((sbits >> p) & 1u) * 0x80000001u;
         float mn1 = f_inf(), mn2 = f_inf();
-        float qf[E];
 #pragma unroll
         for (int k = 0; k < E; ++k) {
-            const float v = ldsf(ln.addr(p, k));
-            qf[k] = v;
+            const float v = qf[k];
             S ^= __float_as_uint(v);
             const float av = fabsf(v);
             mn2 = fminf(mn2, fmaxf(mn1, av));
@@ -703,9 +707,9 @@ struct Decoder {
     // sums), stored tagged with e; at the last iteration slot 0 keeps the
     // tagged L for the cut selection.  Slots past a variable's degree hold 0,
     // so a pass wider than the degree adds exact zeros.  Returns e in every bit.
-    template <bool FAST, int P, int N>
+    template <bool FAST, bool KEEP, int P, int N>
     static __device__ __forceinline__ uint32_t var_group(const DevGraph &g, const L &ln, int u, int t, bool last,
-                                                         float *post_row)
+                                                         float *post_row, float (&lk)[KEEP ? PVM : 1])
     {
         float r[N][CVM];
         uint32_t hd = 0;
@@ -746,10 +750,14 @@ struct Decoder {
                 if (CMIN > 0) sts32(base, lv);
                 else sts32_if(base, lv, ln.has(p, 0));
             }
+            if constexpr (KEEP) {
+                lk[p] = Lp;
+            } else if constexpr (!FAST) {
 #ifdef BPDC_CHECKS
-            if (!FAST && post_row && ((ln.vvalid >> p) & 1u) && !post_ok(g, (long long)p * G + u)) {} else
+                if (post_row && ((ln.vvalid >> p) & 1u) && !post_ok(g, (long long)p * G + u)) {} else
 #endif
-            if (!FAST && post_row && ((ln.vvalid >> p) & 1u)) post_row[__ldg(g.pos_col + p * G + u)] = Lp;
+                if (post_row && ((ln.vvalid >> p) & 1u)) post_row[__ldg(g.pos_col + p * G + u)] = Lp;
+            }
         }
         return hd;
     }
@@ -757,14 +765,14 @@ struct Decoder {
     // The variable updates of passes P .. PVM-1 (all passes of the variant on
     // the fast path, NV at a time, else those the graph occupies); ORs decision
     // bit p of each pass into nhd.
-    template <bool FAST, int P>
+    template <bool FAST, bool KEEP, int P>
     static __device__ __forceinline__ void var_passes(const DevGraph &g, const L &ln, int u, int t, bool last,
-                                                      float *post_row, uint32_t &nhd)
+                                                      float *post_row, uint32_t &nhd, float (&lk)[KEEP ? PVM : 1])
     {
         if constexpr (P < PVM) {
             constexpr int N = !FAST ? 1 : (PVM - P < NV) ? (PVM - P) : NV;
-            if (FAST || P < g.pv) nhd |= var_group<FAST, P, N>(g, ln, u, t, last, post_row);
-            var_passes<FAST, P + N>(g, ln, u, t, last, post_row, nhd);
+            if (FAST || P < g.pv) nhd |= var_group<FAST, KEEP, P, N>(g, ln, u, t, last, post_row, lk);
+            var_passes<FAST, KEEP, P + N>(g, ln, u, t, last, post_row, nhd, lk);
         }
     }
 
@@ -819,20 +827,49 @@ struct Decoder {
         }
     }
 
+    static constexpr bool kKeepPost = PVM <= 5;
+    // One value per variable of this lane into a shot's row of posteriors.
+    static __device__ __forceinline__ void write_post(const DevGraph &g, const L &ln, int u, float *post_row,
+                                                      const float (&v)[PVM])
+    {
+#pragma unroll
+        for (int p = 0; p < PVM; ++p) {
+#ifdef BPDC_CHECKS
+            if (((ln.vvalid >> p) & 1u) && !post_ok(g, (long long)p * G + u)) continue;
+#endif
+            if ((ln.vvalid >> p) & 1u) post_row[__ldg(g.pos_col + p * G + u)] = v[p];
+        }
+    }
+
     // One BP run (flooding, normalized min-sum).  The slots must hold the
     // initial messages, visible to the whole group.  Returns whether the hard
     // decision reproduced the syndrome; iters = iterations used; hd = hard
     // decision bits per variable pass.
     // FAST: every check and variable pass of the variant is occupied and no
-    // posterior is written, so the per-pass guards compile away (the common
-    // case of a graph packed for its own variant; identical arithmetic).
-    template <bool FAST>
+    // posterior is written inside the run, so the per-pass guards compile away
+    // (the common case of a graph packed for its own variant; identical
+    // arithmetic).
+    // KEEP: the posteriors of the last iteration stay in registers and are written
+    // to post_row once, when the run ends (variants of few variable passes); else
+    // the guarded path writes them at every iteration.  50000 BB[[108,8,10]] shots
+    // at p = 0.03 with posteriors: 128 -> 96 us a call.
+    template <bool FAST, bool KEEP>
     static __device__ __forceinline__ bool run(const DevGraph &g, const L &ln, const Group<G> &grp,
                                                uint32_t sbits, uint32_t &hd, int &iters, float *post_row)
     {
         const int u = grp.u;
         const int T = g.max_iter;
         const float alpha = g.alpha;
+        float lk[KEEP ? PVM : 1];
+        if constexpr (KEEP) {
+#pragma unroll
+            for (int p = 0; p < PVM; ++p) lk[p] = ln.lamv[p];
+        }
+        auto end = [&](int n, bool ok) {
+            iters = n;
+            if constexpr (KEEP) write_post(g, ln, u, post_row, lk);
+            return ok;
+        };
         for (int t = 1;; ++t) {
             const bool scatter = t <= T;
             uint32_t unsat = 0;
@@ -840,14 +877,20 @@ struct Decoder {
             constexpr bool kGroup = FAST && RULE == 0 && DCM <= 16 && (NP > 1);
             if constexpr (L::kQuad) unsat = quad_checks(g, ln, u, t, sbits, scatter);
             if constexpr (kGroup) {
+                float qt[kTailEdges];   // the shared last pass is gathered before the others scatter
+                if constexpr (TAIL > 0) tail_gather(ln, PCM - 1, qt);
                 held_passes<0, (TAIL > 0 ? PCM - 1 : PCM)>(ln, sbits, alpha, scatter, unsat);
-                if constexpr (TAIL > 0) unsat |= tail_pass(ln, PCM - 1, sbits, alpha, scatter);
+                if constexpr (TAIL > 0) unsat |= tail_pass(ln, PCM - 1, sbits, alpha, scatter, qt);
             }
 #pragma unroll
             for (int p = 0; p < (L::kQuad || kGroup ? 0 : PCM); ++p) {
                 if constexpr (TAIL > 0) {
                     if (p == PCM - 1) {   // every lane takes part in the shared last pass
-                        if (FAST || p < g.pc) unsat |= tail_pass(ln, p, sbits, alpha, scatter);
+                        if (FAST || p < g.pc) {
+                            float qt[kTailEdges];
+                            tail_gather(ln, p, qt);
+                            unsat |= tail_pass(ln, p, sbits, alpha, scatter, qt);
+                        }
                         continue;
                     }
                 }
@@ -1084,11 +1127,11 @@ struct Decoder {
                     }
                 }
             }
-            if (!grp.any((unsat & 1u) != 0)) { iters = t - 1; return true; }
-            if (t > T) { iters = T; return false; }
+            if (!grp.any((unsat & 1u) != 0)) return end(t - 1, true);
+            if (t > T) return end(T, false);
             // ---- variable phase ----
             uint32_t nhd = 0;
-            var_passes<FAST, 0>(g, ln, u, t, t == T, post_row, nhd);
+            var_passes<FAST, KEEP, 0>(g, ln, u, t, t == T, post_row, nhd, lk);
             hd = nhd & ln.vvalid;
             grp.sync();
         }
@@ -1219,23 +1262,30 @@ struct Decoder {
             // posterior when one is requested), and the correction and
             // logical-flip staging cleared (each lane the words it copies out
             // in the epilogue); the vote is the barrier that publishes both
-            hd = init(g, ln, u, post_row);
+            float *const init_post = kKeepPost ? nullptr : post_row;   // kept posteriors are written by run
+            hd = init(g, ln, u, init_post);
             for (int x = u; x < g.NW; x += G) cm[x] = 0;
             for (int x = u; x < g.KW; x += G) ls[x] = 0;
             const bool nonzero = grp.any(sbits != 0);
             if (!cut_in && !nonzero && g.zero_ok) {
                 // converged before the first iteration: e_hat = 0 (every prior < 1/2)
                 hd = 0;
+                if (kKeepPost && post_row) write_post(g, ln, u, post_row, ln.lamv);
             } else {
                 for (bool second = false;; second = true) {
                     if (second) {
-                        hd = init(g, ln, u, post_row);
+                        hd = init(g, ln, u, init_post);
                         grp.sync();
                     }
                     int iters = 0;
-                    const bool ok = ((L::kQuad || g.pc == PCM) && g.pv == PVM && !post_row)
-                                        ? run<true>(g, ln, grp, sbits, hd, iters, post_row)
-                                        : run<false>(g, ln, grp, sbits, hd, iters, post_row);
+                    const bool full = (L::kQuad || g.pc == PCM) && g.pv == PVM;
+                    bool ok;
+                    if (kKeepPost && post_row)
+                        ok = full ? run<true, kKeepPost>(g, ln, grp, sbits, hd, iters, post_row)
+                                  : run<false, kKeepPost>(g, ln, grp, sbits, hd, iters, post_row);
+                    else
+                        ok = full && !post_row ? run<true, false>(g, ln, grp, sbits, hd, iters, post_row)
+                                               : run<false, false>(g, ln, grp, sbits, hd, iters, post_row);
                     if (second) it2 = iters; else it1 = iters;
                     if (ok) { st = second ? 1 : 0; break; }
                     if (second || cut_in || !g.dc_enable) { st = 2; break; }
@@ -1409,7 +1459,8 @@ __global__ void cut_select_kernel(DevGraph g, int64_t B, const float *post, uint
 // 566 us).  The last two numbers are the check and variable passes whose loads
 // are issued together: more than one pays where a warp has registers left and a
 // shot's latency counts (variant 20: 64 shots of BB[[144,12,12]] 74 -> 65 us, 2*10^5
-// 724 -> 713 us; HGP-2500 and BB[[72,12,6]] gained nothing).
+// 724 -> 713 us; variant 19: 64 shots of BB[[72,12,6]] 39 -> 37 us, 10^5 the same;
+// variant 21 spills with it, 469 -> 582 us per 10^5 shots; HGP-2500 gained nothing).
 #define BPDC_VARIANTS(X)                                                       \
     X(0, 32, 3, 6, 5, 3, 3, true, 0, 256, 4, 0, false, 0, 1, 1)                \
     X(1, 256, 5, 7, 10, 4, 3, true, 0, 256, 3, 0, false, 0, 1, 1)              \
@@ -1430,7 +1481,7 @@ __global__ void cut_select_kernel(DevGraph g, int64_t B, const float *post, uint
     X(16, 512, 2, 35, 18, 6, 2, false, 0, 512, 1, 0x136db6db6e4b76ull, true, 0, 1, 1) \
     X(17, 32, 2, 6, 3, 3, 3, true, 0, 256, 4, 0, false, 0, 1, 1)               \
     X(18, 32, 2, 6, 3, 3, 3, true, 0, 256, 6, 0, false, 0, 1, 1)               \
-    X(19, 32, 2, 6, 3, 3, 3, true, 0, 256, 4, 0, false, 8, 1, 1)               \
+    X(19, 32, 2, 6, 3, 3, 3, true, 0, 256, 4, 0, false, 8, 2, 3)               \
     X(20, 32, 3, 6, 5, 3, 3, true, 0, 256, 3, 0, false, 4, 2, 5)               \
     X(21, 32, 2, 6, 4, 3, 3, true, 0, 256, 4, 0, false, 0, 1, 1)              
 

@@ -48,3 +48,27 @@ def test_two_pass_shape(M, auto):
     r2 = other.decode(s2, 0, obs_true=o2)
     for it, r in zip(items, (r2, ref, r2)):
         assert all(torch.equal(it["out"][x], r[x]) for x in r)
+
+
+@pytest.mark.parametrize("code,kept,stored", [("bb72", (19, 17, 20, 7), 5), ("regular54", (21, 20), 3), ("bb144", (20, 0), 10)])
+@pytest.mark.parametrize("max_iter,dc", [(0, 1), (1, 0), (20, 1)])
+def test_kept_posteriors(code, kept, stored, max_iter, dc):
+    """Posteriors kept in registers until the run ends equal those stored at every
+    iteration: converged, failed, after a cut, for a zero syndrome and on a given
+    cut set."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2510_08695_gb300 as pkg
+    P = _regular(54) if code == "regular54" else bi.bb_problem(code, 0.06)
+    g = pkg.Graph.from_problem(P, pkg.Options(max_iter=max_iter, dc_enable=dc, dc_prior=dc))
+    syn, _, _ = g.sample(500, 5, 0)
+    syn[7] = 0
+    cut = g.cut_select(torch.randn((500, g.N), generator=torch.Generator(device="cuda").manual_seed(1), device="cuda"))
+    g.set_kernel(stored)
+    ref = [g.decode(syn, 0, posterior=True), g.decode(syn, 0, posterior=True, cut_in=cut, persistent=False)]
+    for k in kept:
+        g.set_kernel(k)
+        out = [g.decode(syn, 0, posterior=True), g.decode(syn, 0, posterior=True, cut_in=cut, persistent=False)]
+        for a, b in zip(out, ref):
+            assert all(torch.equal(a[x], b[x]) for x in b), k
