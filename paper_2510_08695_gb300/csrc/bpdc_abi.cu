@@ -88,6 +88,7 @@ struct DeviceGuard {
 };
 
 constexpr int kRing = BPDC_MAX_INFLIGHT;
+constexpr size_t kWorkStride = 128;   // bytes between work counters
 constexpr int64_t kHostChunk = 262144;   // default shots per piece of bpdc_decode_host
 constexpr int kMaxBatches = 32;
 constexpr int kMaxSmemPerBlock = 227 * 1024;
@@ -451,6 +452,9 @@ int plan_and_upload(bpdc_graph_s *g, int want_G, int want_id = -1)
     const size_t o_rmask = put(blob, rmask), o_cchk = put(blob, cchk);
     const size_t o_wts = put(blob, P.wts);
     const size_t o_err = put(blob, std::vector<int32_t>(4, 0));
+    // work counters of the ring's slots, a cache line each: every launch leaves
+    // its counter at 0 for the next one on its slot
+    const size_t o_work = put(blob, std::vector<char>((size_t)kRing * kWorkStride, 0));
     void *arena = nullptr;
     e = lib_malloc(&arena, blob.size());
     if (e != cudaSuccess) return fail(BPDC_ERR_OOM, "cudaMalloc of %zu bytes: %s", blob.size(), cudaGetErrorString(e));
@@ -503,6 +507,7 @@ int plan_and_upload(bpdc_graph_s *g, int want_G, int want_id = -1)
     d.n_d_ent = (int64_t)P.d_ent.size();
     d.n_wts = (int64_t)P.wts.size();
 #endif
+    for (int s = 0; s < kRing; ++s) g->ring[s].work = (unsigned long long *)(base + o_work + (size_t)s * kWorkStride);
     g->variant = vid;
     g->groups_per_block = gpb;
     g->blocks_per_sm = bps;
@@ -513,23 +518,17 @@ int plan_and_upload(bpdc_graph_s *g, int want_G, int want_id = -1)
 
 int ring_init(bpdc_graph_s *g)
 {
-    const size_t per = sizeof(BatchDesc) * kMaxBatches + 256;
+    const size_t per = sizeof(BatchDesc) * kMaxBatches;
     cudaError_t e = lib_malloc(&g->ring_mem, per * kRing);
     if (e != cudaSuccess) return fail(BPDC_ERR_OOM, "ring allocation: %s", cudaGetErrorString(e));
     e = lib_malloc_host(&g->ring_host, sizeof(BatchDesc) * kMaxBatches * kRing);
     if (e != cudaSuccess) return fail(BPDC_ERR_OOM, "pinned ring allocation: %s", cudaGetErrorString(e));
     for (int s = 0; s < kRing; ++s) {
-        char *b = (char *)g->ring_mem + per * s;
-        g->ring[s].work = (unsigned long long *)b;
-        g->ring[s].dev_desc = (BatchDesc *)(b + 256);
+        g->ring[s].dev_desc = (BatchDesc *)((char *)g->ring_mem + per * s);
         g->ring[s].host_desc = (BatchDesc *)g->ring_host + (size_t)kMaxBatches * s;
         e = cudaEventCreateWithFlags(&g->ring[s].done, cudaEventDisableTiming);
         if (e != cudaSuccess) return cuda_fail(e, "event creation");
     }
-    // every launch leaves its work counter at 0 for the next one on its slot
-    e = cudaMemset2D(g->ring_mem, per, 0, sizeof(unsigned long long), kRing);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
-    if (e != cudaSuccess) return cuda_fail(e, "work counters");
     return BPDC_OK;
 }
 
