@@ -1137,10 +1137,21 @@ struct Decoder {
         }
     }
 
+    // ONE: a launch of one batch, whose descriptor is read from the kernel's
+    // parameters in place: no pointer to it is held across the iterations (the
+    // registers it takes were spilled) and a shot's fields come from the constant
+    // bank.  10^5 phenomenological BB[[72,12,6]] shots at p = 0.006 1.50 -> 1.25 ms,
+    // BB[[144,12,12]] at p = 0.002 4.49 -> 4.05 ms; distance-7 surface code 2.75 ->
+    // 2.63 ms.
+    template <bool ONE>
     static __device__ void decode(const LaunchDesc &ld, uint32_t *region, const Group<G> &grp, int gib)
     {
         const int u = grp.u;
-        const BatchDesc *const batches = ld.batches ? ld.batches : ld.own;
+        const BatchDesc *const batches = ONE || !ld.batches ? ld.own : ld.batches;
+        auto desc = [&](int i) -> const BatchDesc & {
+            if constexpr (ONE) return ld.own[0];
+            else return batches[i];
+        };
         L ln;
         // little state lives across the iterations (the loop needs the
         // registers): shot indices are 32-bit (a launch holds fewer than 2^32
@@ -1197,25 +1208,25 @@ struct Decoder {
             if ((int64_t)w >= ld.total) break;
             if (w < bfirst || w >= bend) {
                 if (u == 0) {
-                    if (bi >= 0 && batches[bi].counters)
-                        for (int x = 0; x < 4; ++x) atomicAdd(batches[bi].counters + x, cnt[x]);
+                    if (bi >= 0 && desc(bi).counters)
+                        for (int x = 0; x < 4; ++x) atomicAdd(desc(bi).counters + x, cnt[x]);
                     cnt[0] = cnt[1] = cnt[2] = cnt[3] = 0;
                 }
-                int lo = 0, hi = ld.n_batches - 1;
+                int lo = 0, hi = ONE ? 0 : ld.n_batches - 1;
                 while (lo < hi) {  // last batch with first <= w
                     const int mid = (lo + hi + 1) >> 1;
-                    if (batches[mid].first <= (int64_t)w) lo = mid; else hi = mid - 1;
+                    if (desc(mid).first <= (int64_t)w) lo = mid; else hi = mid - 1;
                 }
-                const DevGraph &gnew = batches[lo].g;
-                if (bi < 0 || gnew.chk_idx != batches[bi].g.chk_idx || gnew.lam != batches[bi].g.lam) {
+                const DevGraph &gnew = desc(lo).g;
+                if (bi < 0 || gnew.chk_idx != desc(bi).g.chk_idx || gnew.lam != desc(bi).g.lam) {
                     ln.load(gnew, u, slot_base, inf_word);
                     lam_dirty = false;
                 }
                 bi = lo;
-                bfirst = (uint32_t)batches[bi].first;
-                bend = bfirst + (uint32_t)batches[bi].B;
+                bfirst = (uint32_t)desc(bi).first;
+                bend = bfirst + (uint32_t)desc(bi).B;
             }
-            const BatchDesc &bd = batches[bi];
+            const BatchDesc &bd = desc(bi);
             // the graph's fields are read where they are used (L1 hits), not
             // copied per shot: a copy of the whole descriptor took registers
             // and stack from the iterations (2-10 % slower)
@@ -1379,13 +1390,13 @@ struct Decoder {
                 cnt[3] += ran_dc ? 1 : 0;
             }
         }
-        if (bi >= 0 && u == 0 && batches[bi].counters)
-            for (int x = 0; x < 4; ++x) atomicAdd(batches[bi].counters + x, cnt[x]);
+        if (bi >= 0 && u == 0 && desc(bi).counters)
+            for (int x = 0; x < 4; ++x) atomicAdd(desc(bi).counters + x, cnt[x]);
     }
 };
 
 template <int G, int PCM, int DCM, int PVM, int CVM, int CMIN, bool RC, int RULE, int BLOCK, int MINB,
-          uint64_t PROF, bool TAB, int TAIL, int NP, int NV>
+          uint64_t PROF, bool TAB, int TAIL, int NP, int NV, bool ONE>
 __global__ void __launch_bounds__(BLOCK, MINB) decode_kernel(const __grid_constant__ LaunchDesc ld, int region_words)
 {
     extern __shared__ uint32_t smem[];
@@ -1404,7 +1415,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) decode_kernel(const __grid_consta
         grp.leader = 0;
     }
     uint32_t *region = smem + (size_t)gib * region_words;
-    Decoder<G, PCM, DCM, PVM, CVM, CMIN, RC, RULE, PROF, TAB, TAIL, NP, NV>::decode(ld, region, grp, gib);
+    Decoder<G, PCM, DCM, PVM, CVM, CMIN, RC, RULE, PROF, TAB, TAIL, NP, NV>::template decode<ONE>(ld, region, grp, gib);
 }
 
 // Cut selection alone, one block per shot (same selection code as the fused kernel).
@@ -1510,11 +1521,20 @@ bool check_status(int *site, long long *index)
 bool check_status(int *, long long *) { return false; }
 #endif
 
-static const void *variant_fn(int id)
+// Variants with a second instance for launches of one batch (Decoder::decode): the
+// automatic choices that it makes faster.  Not variants 15 and 19: HGP-2500 30001
+// shots gain at p = 0.02 (2.83 -> 2.75 ms) but lose at 0.06 (14.75 -> 14.88 ms), where
+// the workload's time is, and BB[[72,12,6]] is 1.64 ms either way; nor those that no
+// rule chooses first (each instance costs build time).
+static constexpr bool one_batch_form(int id) { return id == 3 || id == 11 || id == 16 || id == 20 || id == 21; }
+
+static const void *variant_fn(int id, bool one)
 {
     switch (id) {
 #define X(id, G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV) \
-    case id: return (const void *)decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV>;
+    case id:                                                                                        \
+        return one ? (const void *)decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV, one_batch_form(id)> \
+                   : (const void *)decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV, false>;
         BPDC_VARIANTS(X)
 #undef X
     default: return nullptr;
@@ -1526,7 +1546,7 @@ static const void *variant_fn(int id)
 // created later never lowers it under a larger one that is still in use.
 cudaError_t variant_attributes(int id, int smem_bytes, int *blocks_per_sm, int *regs)
 {
-    const void *fn = variant_fn(id);
+    const void *fn = variant_fn(id, false);
     if (!fn) return cudaErrorInvalidValue;
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1544,6 +1564,8 @@ cudaError_t variant_attributes(int id, int smem_bytes, int *blocks_per_sm, int *
     int &lim = limit[std::make_pair(dev, id)];
     if (smem_bytes > lim) {
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+        if (e == cudaSuccess && one_batch_form(id))
+            e = cudaFuncSetAttribute(variant_fn(id, true), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
         if (e != cudaSuccess) return e;
         lim = smem_bytes;
     }
@@ -1563,11 +1585,16 @@ cudaError_t launch_variant(int id, const LaunchDesc &ld, int grid, int groups, i
 {
     const int region = smem_bytes / 4 / (kVariants[id].block_threads / kVariants[id].G);
     const int threads = groups * kVariants[id].G, smem = groups * region * 4;
+    const bool one = ld.n_batches == 1 && !ld.batches;
     switch (id) {
 #define X(id, G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV)                          \
     case id:                                                                                        \
-        decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV>                  \
-            <<<grid, threads, smem, s>>>(ld, region);                                               \
+        if (one)                                                                                    \
+            decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV, one_batch_form(id)> \
+                <<<grid, threads, smem, s>>>(ld, region);                                           \
+        else                                                                                        \
+            decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV, false>       \
+                <<<grid, threads, smem, s>>>(ld, region);                                           \
         return cudaGetLastError();
         BPDC_VARIANTS(X)
 #undef X
