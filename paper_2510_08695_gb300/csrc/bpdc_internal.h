@@ -223,7 +223,7 @@ struct WbpArgs {
     float *post;                 // [B][T][N] or null
     float *S;                    // [B][T][E] sum of phi over the other edges of the check, with r's sign
     const float *gpost;          // [B][T][N] adjoint of the posteriors (backward)
-    float *part;                 // [blocks][2: hi, lo][2][T][E] partial gradients (backward)
+    float *part;                 // [blocks][2: high, low word][2][T][E] partial gradients, FP64 (backward)
 };
 size_t wbp_smem_backward(int E, int k, int warps);
 cudaError_t launch_wbp_forward(const DevGraph &g, const WbpArgs &a, cudaStream_t s);

@@ -27,13 +27,13 @@
 // rounding, do not depend on the launch.
 //
 // Gradients are summed over shots in a fixed order: the shots of a block (4 to 8)
-// in shared memory at each iteration, the blocks' sums by a second kernel.  Sums
-// are pairs hi + lo of floats (error-free two-sum): FP64 adds run at a 64th of the
-// FP32 rate here, and a store of every shot's gradients was 283 MB a call.
+// in shared memory at each iteration (sum64), the blocks' sums by a second kernel,
+// both in FP64: partial sums of gradients that cancel may lie far above the total, up
+// to beyond the float range.  A store of every shot's gradients was 283 MB a call.
 //
 // BB[[144,12,12]], T = 20, 4096 shots: forward 545 -> 299 us (issue 79 %), adjoint
-// 2540 -> 503 us (11 900 -> 5050 warp instructions per shot and iteration, issue
-// 70 %), sum of the gradients 790 -> 25 us.
+// with the sum of the gradients 3330 -> 565 us a call (11 900 -> about 5050 warp
+// instructions per shot and iteration).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -63,6 +63,9 @@ __device__ __forceinline__ float with_sign(float mag, bool neg)
 }
 __device__ __forceinline__ bool sign_of(float x) { return (__float_as_uint(x) >> 31) != 0u; }
 
+// Most shots of a block.
+constexpr int most_shots(int G) { return 1024 / G < 8 ? 1024 / G : 8; }
+
 // The G threads that work on a shot; named barrier 1 + index of the shot in the block.
 template <int G>
 __device__ __forceinline__ void team_sync(int team)
@@ -70,18 +73,41 @@ __device__ __forceinline__ void team_sync(int team)
     asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(G) : "memory");
 }
 
-// A sum kept as hi + lo: lo collects the exact rounding errors of hi (two-sum),
-// which carries some 48 bits; with an overflow or a NaN only hi counts.
-struct Sum2 {
-    float hi = 0.0f, lo = 0.0f;
-    __device__ __forceinline__ void add(float x)
-    {
-        const float s = hi + x, b = s - hi;
-        lo += (hi - (s - b)) + (x - b);
-        hi = s;
+// The sum of n <= MOST floats x[0], x[stride], ... to more than FP64's 53 bits: a
+// float that collects the sum, one that collects its exact rounding errors (two-sum)
+// and one for theirs, added up in FP64 at the end.  FP64 runs at a 64th of the FP32
+// rate here: with an FP64 add for each of the 71 million terms of 4096 BB[[144,12,12]]
+// shots, T = 20, a backward call takes 599 us, with this form 565 (533 with two floats,
+// some 48 bits and the range of one).  Sums that leave the float range on the way, or
+// hold an infinity or a NaN, are taken again term by term in FP64.
+__device__ __forceinline__ void two_sum(float &s, float x, float &err)
+{
+    const float t = s + x, b = t - s;
+    err = (s - (t - b)) + (x - b);
+    s = t;
+}
+template <int MOST>
+__device__ __forceinline__ double sum64(const float *x, int n, size_t stride)
+{
+    float v[MOST];
+#pragma unroll
+    for (int w = 0; w < MOST; ++w) v[w] = w < n ? x[w * stride] : 0.0f;
+    float a = v[0], b, c = 0.0f;
+    two_sum(a, v[1], b);
+#pragma unroll
+    for (int w = 2; w < MOST; ++w) {
+        if (w >= n) break;
+        float e, f;
+        two_sum(a, v[w], e);
+        two_sum(b, e, f);
+        c += f;
     }
-    __device__ __forceinline__ float value() const { return isfinite(hi) ? hi + lo : hi; }
-};
+    // where a is not finite, neither is its error b
+    if (isfinite(b + c)) return (double)a + ((double)b + (double)c);
+    double s = 0.0;
+    for (int w = 0; w < n; ++w) s += (double)x[w * stride];
+    return s;
+}
 
 // In place over the edges of every variable (lanes over variables; m-th edge of
 // variable j in c_edget[m * N + j]): out(j, base, pre_m + suf_m) with pre_m / suf_m
@@ -277,17 +303,14 @@ __global__ void __launch_bounds__(G == 64 ? 512 : 1024, G == 64 ? 4 : 2) wbp_bac
                 const int e = second ? n - E : n;
                 const float *src = sm + (second ? E : 3 * E) + e;
                 const size_t at = (size_t)((second ? T : 0) + t) * E + e;
-                Sum2 s;
-                if (base != (int64_t)blockIdx.x * W) {
-                    s.hi = part[at];
-                    s.lo = part[nw + at];
-                }
-                for (int w = 0; w < shots; ++w) s.add(src[(size_t)w * 4 * E]);
+                double s = sum64<most_shots(G)>(src, shots, (size_t)4 * E);
+                if (base != (int64_t)blockIdx.x * W)
+                    s += __hiloint2double(__float_as_int(part[at]), __float_as_int(part[nw + at]));
                 if (direct) {
-                    grad_w[at] = s.value();
+                    grad_w[at] = (float)s;
                 } else {
-                    part[at] = s.hi;
-                    part[nw + at] = s.lo;
+                    part[at] = __int_as_float(__double2hiint(s));
+                    part[nw + at] = __int_as_float(__double2loint(s));
                 }
             }
         }
@@ -298,28 +321,23 @@ __global__ void __launch_bounds__(G == 64 ? 512 : 1024, G == 64 ? 4 : 2) wbp_bac
 // Sum of the blocks' partial sums in block order: 32 weights x 8 runs of blocks.
 __global__ void __launch_bounds__(256) wbp_reduce_kernel(const float *part, int blocks, int64_t nw, float *out)
 {
-    __shared__ float hi[8][32], lo[8][32];
+    __shared__ double sums[8][32];
     const int lane = threadIdx.x & 31, run = threadIdx.x >> 5;
     const int64_t w = (int64_t)blockIdx.x * 32 + lane;
     const int per = (blocks + 7) / 8, b1 = min(blocks, (run + 1) * per);
-    Sum2 s;
+    double s = 0.0;
     if (w < nw)
         for (int b = run * per; b < b1; ++b) {
-            s.add(part[(size_t)b * 2 * nw + w]);
-            s.lo += part[((size_t)b * 2 + 1) * nw + w];
+            const float *p = part + (size_t)b * 2 * nw + w;
+            s += __hiloint2double(__float_as_int(p[0]), __float_as_int(p[nw]));
         }
-    hi[run][lane] = s.hi;
-    lo[run][lane] = s.lo;
+    sums[run][lane] = s;
     __syncthreads();
     if (run == 0 && w < nw) {
-        for (int k = 1; k < 8; ++k) {
-            s.add(hi[k][lane]);
-            s.lo += lo[k][lane];
-        }
-        out[w] = s.value();
+        for (int k = 1; k < 8; ++k) s += sums[k][lane];
+        out[w] = (float)s;
     }
 }
-
 
 // Threads per shot: 64 where that gives every SM 16 warps (of the shots an SM gets
 // and has memory for in the adjoint), else 256.  BB[[144,12,12]], T = 20, forward /
@@ -357,7 +375,7 @@ int shots_per_block(int64_t B, int least, int most)
 // shots where that is short.
 void backward_plan(int64_t B, int E, int T, int G, int *shots, int64_t *blocks)
 {
-    const int most = (int)std::min<size_t>(std::min(8, 1024 / G), kMaxWbpSmem / ((size_t)16 * E));
+    const int most = (int)std::min<size_t>(most_shots(G), kMaxWbpSmem / ((size_t)16 * E));
     const int64_t room = std::max<int64_t>(1, B * (T + 1) / ((int64_t)4 * T));
     int w = shots_per_block(B, std::min(4, most), most);
     while (w < most && (B + w - 1) / w > room) ++w;
@@ -381,7 +399,7 @@ cudaError_t launch_wbp_forward(const DevGraph &g, const WbpArgs &a, cudaStream_t
     if (a.B <= 0) return cudaSuccess;
     if (a.E > kWbpMaxEdges) return cudaErrorInvalidValue;
     const int G = team_size(a.B, a.E);
-    const int w = shots_per_block(a.B, 1, std::min(8, 1024 / G));
+    const int w = shots_per_block(a.B, 1, most_shots(G));
     const size_t smem = (size_t)w * a.E * sizeof(float);
     const int grid = (int)std::min<int64_t>((a.B + w - 1) / w, 152 * 32);
     auto go = [&](auto kernel) {
