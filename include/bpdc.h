@@ -263,16 +263,17 @@ int bpdc_decode_host(const bpdc_batch *batches, int32_t n_batches, int64_t chunk
  *     launched.
  *   - The first call on a device looks up the array's device address; make
  *     that first call before any stream capture on that device.
- *   - Every call reuses the same array (each decode leaves the work counter at
- *     zero for the next).  Calls whose launches overlap on the GPU, e.g. on
- *     two streams, race on it: keep such calls ordered on one stream.
- *   - The call issues kernel launches and nothing else: the decode kernel, which
- *     carries up to four batch descriptors in its parameters, and for more
- *     batches a setup kernel before it that receives them as parameters and
- *     writes them into the array (both once more where variants 20 and 21 are
- *     mixed).  It can therefore be captured into a CUDA graph (after a first
- *     uncaptured call on the device); each replay decodes whatever the captured
- *     syndrome buffers hold into the captured output buffers.
+ *   - Every call reuses the same array.  Calls whose launches overlap on the
+ *     GPU, e.g. on two streams, race on it and give wrong results: keep such
+ *     calls ordered on one stream.  Later calls are not affected.
+ *   - The call issues kernel launches and nothing else: a setup kernel that
+ *     clears the work counter and, where there are more than four batches,
+ *     receives their descriptors as parameters and writes them into the array,
+ *     then the decode kernel, which carries up to four in its own parameters
+ *     (both once more where variants 20 and 21 are mixed).  It can therefore be
+ *     captured into a CUDA graph (after a first uncaptured call on the device);
+ *     each replay decodes whatever the captured syndrome buffers hold into the
+ *     captured output buffers.
  * Results equal those of bpdc_decode_multi on the same batches. */
 int bpdc_decode_multi_noalloc(const bpdc_batch *batches, int32_t n_batches, void *stream);
 
