@@ -200,7 +200,7 @@ def phenomenological_leg(args, pkg, torch, stream, peak_gbs) -> dict:
     # the probe: 10^5 shots of the p = 0.010 point, enough that the few shots
     # running all 1000 + 1000 iterations do not decide the launch's length alone
     probe = items[-1]
-    tune = autotune(probe["graph"], probe["syndromes"][:min(100000, spp)].contiguous(), 0)
+    tune = autotune(probe["graph"], probe["syndromes"][:min(100000, spp)].contiguous(), 0, batches=len(items))
     for it in items:
         it["graph"].set_kernel(tune["best"])
     vid = tune["best"]
@@ -447,7 +447,8 @@ def main():
     for code in sorted({b["code"] for b in batches} if args.kernel is None else ()):
         probe = max((b for b in batches if b["code"] == code), key=lambda b: b["p"])
         n = min(20000, spp)
-        res = autotune(probe["graph"], probe["syndromes"][:n].contiguous(), probe["shot_offset"])
+        res = autotune(probe["graph"], probe["syndromes"][:n].contiguous(), probe["shot_offset"],
+                       batches=sum(b["code"] == code for b in batches))
         for b in batches:
             if b["code"] == code:
                 b["graph"].set_kernel(res["best"])

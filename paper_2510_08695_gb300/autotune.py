@@ -5,7 +5,8 @@ checks and variables each thread owns, the row and column weights they are
 specialised for, and their register budget (resident blocks per SM).  For a
 graph the autotuner times every variant that accepts it on a sample of shots
 (CUDA events on the current stream, after a warm-up launch) and keeps the
-fastest; the graph's automatically chosen variant stays unless another is
+fastest for launches of the wanted number of batches (some variants have a
+kernel of their own for launches of one batch); the graph's automatically chosen variant stays unless another is
 more than ``margin`` faster, so that near-ties do not flip between runs.
 Results are identical for every variant; only the speed differs.
 """
@@ -21,9 +22,25 @@ def choose(times: dict, incumbent: int, margin: float = 0.02) -> int:
     return best
 
 
+def launcher(graph, syndromes, shot_offset: int, out: dict, persistent: bool, batches: int):
+    """The call that autotune times: one ``decode`` of the sample, or one
+    ``decode_multi`` (always persistent) of the sample cut into ``batches``."""
+    from . import _bpdc
+    B = int(syndromes.shape[0])
+    n = min(batches, B)
+    if n <= 1:
+        return lambda: graph.decode(syndromes, shot_offset, out=out, persistent=persistent)
+    cuts = [B * i // n for i in range(n + 1)]
+    items = [dict(graph=graph, syndromes=syndromes[a:b], shot_offset=shot_offset + a,
+                  out={k: v[a:b] for k, v in out.items()}) for a, b in zip(cuts, cuts[1:])]
+    return lambda: _bpdc.decode_multi(items)
+
+
 def autotune(graph, syndromes, shot_offset: int = 0, reps: int = 2, persistent: bool = True,
-             verbose: bool = False, margin: float = 0.02) -> dict:
-    """Selects the fastest kernel variant for ``graph`` on ``syndromes``.
+             verbose: bool = False, margin: float = 0.02, batches: int = 1) -> dict:
+    """Selects the fastest kernel variant for ``graph`` on ``syndromes``, decoded
+    as one batch or, for graphs that ``decode_multi`` will take in lists, cut into
+    ``batches`` of one list.
 
     Returns ``{"best": kernel_id, "ms": {kernel_id: ms per decode}}``.
     """
@@ -34,13 +51,14 @@ def autotune(graph, syndromes, shot_offset: int = 0, reps: int = 2, persistent: 
     for k in graph.kernels():
         graph.set_kernel(k)
         out = graph.alloc_outputs(B, iterations=False, logical=True)
-        graph.decode(syndromes, shot_offset, out=out, persistent=persistent)
+        run = launcher(graph, syndromes, shot_offset, out, persistent, batches)
+        run()
         torch.cuda.synchronize()
         e0 = torch.cuda.Event(enable_timing=True)
         e1 = torch.cuda.Event(enable_timing=True)
         e0.record()
         for _ in range(reps):
-            graph.decode(syndromes, shot_offset, out=out, persistent=persistent)
+            run()
         e1.record()
         torch.cuda.synchronize()
         times[k] = e0.elapsed_time(e1) / reps
