@@ -351,8 +351,8 @@ int bpdc_measure_smem_peak(int32_t device, int32_t reps, double *bytes_per_secon
  * no result depends on it.  Calls are stream-ordered and asynchronous.  Errors:
  * BPDC_ERR_INVALID_ARG (NULL buffers, T outside [1, 1000], ckpt_every
  * outside [1, T], clip outside (0, 30], workspace too small),
- * BPDC_ERR_UNSUPPORTED (row/column weights, or more edges than the adjoint's
- * shared memory holds), BPDC_ERR_CUDA. */
+ * BPDC_ERR_UNSUPPORTED (row/column weights, or more than 3632 edges, whatever
+ * the interval), BPDC_ERR_CUDA. */
 
 /* Makes bpdc_decode / bpdc_decode_multi run weighted BP with learned weights
  * (host float [2][T][E], the layout above; copied) inside BP+DC: decoding

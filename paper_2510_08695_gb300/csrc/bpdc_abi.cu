@@ -1232,8 +1232,8 @@ static int wbp_prepare(bpdc_graph_t g, int64_t B, const uint32_t *syndromes, con
         return fail(BPDC_ERR_UNSUPPORTED, "weighted BP needs row weights in [2, %d] and column weights <= %d",
                     kWbpMaxRow, kWbpMaxCol);
     const int E = (int)g->H.col.size();
-    if (wbp_smem_backward(E, ckpt_every, 1) > kMaxWbpSmem)
-        return fail(BPDC_ERR_UNSUPPORTED, "graph too large for the weighted-BP adjoint (%d edges)", E);
+    if (E > kWbpMaxEdges)
+        return fail(BPDC_ERR_UNSUPPORTED, "weighted BP takes graphs of at most %d edges (got %d)", kWbpMaxEdges, E);
     size_t need = 0;
     bpdc_wbp_workspace_size(g, B, T, ckpt_every, &need);
     if (B > 0 && (!workspace || workspace_bytes < need))

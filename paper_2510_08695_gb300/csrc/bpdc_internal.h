@@ -213,6 +213,8 @@ cudaError_t launch_cut_select(const DevGraph &g, int64_t B, const float *post, u
 constexpr int kWbpMaxRow = 16;
 constexpr int kWbpMaxCol = 8;
 constexpr size_t kMaxWbpSmem = 227 * 1024;
+// Most edges: four shots of the adjoint (four floats an edge each) fit a block's memory.
+constexpr int kWbpMaxEdges = (int)(kMaxWbpSmem / (4 * 4 * sizeof(float)));
 struct WbpArgs {
     int64_t B;
     int E, T;                    // edges, iterations
@@ -225,7 +227,6 @@ struct WbpArgs {
     const float *gpost;          // [B][T][N] adjoint of the posteriors (backward)
     float *part;                 // [blocks][2: high, low word][2][T][E] partial gradients, FP64 (backward)
 };
-size_t wbp_smem_backward(int E, int k, int warps);
 cudaError_t launch_wbp_forward(const DevGraph &g, const WbpArgs &a, cudaStream_t s);
 cudaError_t launch_wbp_backward(const DevGraph &g, const WbpArgs &a, float *grad_w, cudaStream_t s);
 

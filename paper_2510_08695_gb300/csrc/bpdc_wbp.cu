@@ -47,8 +47,6 @@ namespace {
 
 constexpr float kQmin = 1e-6f;
 constexpr int kNoEdge16 = 0xFFFF;
-// Most edges (as ever: the message arrays of eight shots fit a block's memory).
-constexpr int kWbpMaxEdges = (int)(kMaxWbpSmem / (8 * 2 * sizeof(float)));
 
 __device__ __forceinline__ float wphi(float x) { return log1pf(2.0f / expm1f(x)); }
 
@@ -391,8 +389,6 @@ cudaError_t allow_smem(K kernel, size_t smem)
 }
 
 }  // namespace
-
-size_t wbp_smem_backward(int E, int k, int warps) { return (size_t)warps * (2 * k + 2) * E * sizeof(float); }
 
 cudaError_t launch_wbp_forward(const DevGraph &g, const WbpArgs &a, cudaStream_t s)
 {
