@@ -701,15 +701,30 @@ struct Decoder {
         return hd & ln.vvalid;
     }
 
+    // What the guarded path reads of the descriptor at every pass is read once a run
+    // instead: its stores of posteriors may alias the descriptor, so each pass loaded
+    // it again, and by the slower generic loads since a descriptor may lie in the
+    // kernel's parameters.  The number of check passes for the min-sum variants whose
+    // posteriors are stored there (see kKeepPost); the number of variable passes and the
+    // column table too but for the slot profiles, whose fast path that slows (variant
+    // 15: 2.57 -> 2.60 ms per 5000 HGP-2500 shots at p = 0.06).  Variant 12 spills with
+    // any of it, variant 19 loses 1 % in lists.
+    // With posteriors: variant 15 4.09 -> 4.02 ms, variant 3 (in a list) 2.05 -> 1.73 per
+    // 50000 phenomenological shots at p = 0.004, variant 10 2.37 -> 1.95.  Without: five
+    // rates of 20000 phenomenological BB[[72,12,6]] shots, which leave variant 3 passes
+    // over, 1.59 -> 1.37 ms; of BB[[144,12,12]] 12.2 -> 11.9.
+    static constexpr bool kHoldChecks = RULE == 0 && PVM > 5, kHoldTables = kHoldChecks && PROF == 0;
+
     // Variable update at pass P (CVP = L::cv(P) slots per variable): the
     // posterior L = lambda + sum r, the hard decision e = [L <= 0] (Eq. 4) and
     // the extrinsic messages q = lambda + the other r (prefix and suffix
     // sums), stored tagged with e; at the last iteration slot 0 keeps the
     // tagged L for the cut selection.  Slots past a variable's degree hold 0,
-    // so a pass wider than the degree adds exact zeros.  Returns e in every bit.
+    // so a pass wider than the degree adds exact zeros.  Returns the decision bits.
     template <bool FAST, bool KEEP, int P, int N>
     static __device__ __forceinline__ uint32_t var_group(const DevGraph &g, const L &ln, int u, int t, bool last,
-                                                         float *post_row, float (&lk)[KEEP ? PVM : 1])
+                                                         float *post_row, const int32_t *pos_col,
+                                                         float (&lk)[KEEP ? PVM : 1])
     {
         float r[N][CVM];
         uint32_t hd = 0;
@@ -756,7 +771,8 @@ struct Decoder {
 #ifdef BPDC_CHECKS
                 if (post_row && ((ln.vvalid >> p) & 1u) && !post_ok(g, (long long)p * G + u)) {} else
 #endif
-                if (post_row && ((ln.vvalid >> p) & 1u)) post_row[__ldg(g.pos_col + p * G + u)] = Lp;
+                if (post_row && ((ln.vvalid >> p) & 1u))
+                    post_row[__ldg((kHoldTables ? pos_col : g.pos_col) + p * G + u)] = Lp;
             }
         }
         return hd;
@@ -767,12 +783,14 @@ struct Decoder {
     // bit p of each pass into nhd.
     template <bool FAST, bool KEEP, int P>
     static __device__ __forceinline__ void var_passes(const DevGraph &g, const L &ln, int u, int t, bool last,
-                                                      float *post_row, uint32_t &nhd, float (&lk)[KEEP ? PVM : 1])
+                                                      float *post_row, int pv, const int32_t *pos_col,
+                                                      uint32_t &nhd, float (&lk)[KEEP ? PVM : 1])
     {
         if constexpr (P < PVM) {
             constexpr int N = !FAST ? 1 : (PVM - P < NV) ? (PVM - P) : NV;
-            if (FAST || P < g.pv) nhd |= var_group<FAST, KEEP, P, N>(g, ln, u, t, last, post_row, lk);
-            var_passes<FAST, KEEP, P + N>(g, ln, u, t, last, post_row, nhd, lk);
+            if (FAST || P < (kHoldTables ? pv : g.pv))
+                nhd |= var_group<FAST, KEEP, P, N>(g, ln, u, t, last, post_row, pos_col, lk);
+            var_passes<FAST, KEEP, P + N>(g, ln, u, t, last, post_row, pv, pos_col, nhd, lk);
         }
     }
 
@@ -860,6 +878,8 @@ struct Decoder {
         const int u = grp.u;
         const int T = g.max_iter;
         const float alpha = g.alpha;
+        const int pc = g.pc, pv = g.pv;
+        const int32_t *const pos_col = g.pos_col;
         float lk[KEEP ? PVM : 1];
         if constexpr (KEEP) {
 #pragma unroll
@@ -886,7 +906,7 @@ struct Decoder {
             for (int p = 0; p < (L::kQuad || kGroup ? 0 : PCM); ++p) {
                 if constexpr (TAIL > 0) {
                     if (p == PCM - 1) {   // every lane takes part in the shared last pass
-                        if (FAST || p < g.pc) {
+                        if (FAST || p < (kHoldChecks ? pc : g.pc)) {
                             float qt[kTailEdges];
                             tail_gather(ln, p, qt);
                             unsat |= tail_pass(ln, p, sbits, alpha, scatter, qt);
@@ -897,7 +917,7 @@ struct Decoder {
                 // on the fast path every check pass but the last is full, and
                 // lanes without a check in the last pass skip it (their edges
                 // all point at the +inf word, which keeps its value)
-                if (FAST ? (p < PCM - 1 || ((ln.cvalid >> p) & 1u)) : p < g.pc) {
+                if (FAST ? (p < PCM - 1 || ((ln.cvalid >> p) & 1u)) : p < (kHoldChecks ? pc : g.pc)) {
                     const bool live = (FAST && p < PCM - 1) || ((ln.cvalid >> p) & 1u);
                     // rows of up to 16 edges keep the gathered q in registers for
                     // the scatter; longer rows read each q again before
@@ -1131,7 +1151,7 @@ struct Decoder {
             if (t > T) return end(T, false);
             // ---- variable phase ----
             uint32_t nhd = 0;
-            var_passes<FAST, KEEP, 0>(g, ln, u, t, t == T, post_row, nhd, lk);
+            var_passes<FAST, KEEP, 0>(g, ln, u, t, t == T, post_row, pv, pos_col, nhd, lk);
             hd = nhd & ln.vvalid;
             grp.sync();
         }
