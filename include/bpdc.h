@@ -267,9 +267,9 @@ int bpdc_decode_host(const bpdc_batch *batches, int32_t n_batches, int64_t chunk
  *     GPU, e.g. on two streams, race on it and give wrong results: keep such
  *     calls ordered on one stream.  Later calls are not affected.
  *   - The call issues kernel launches and nothing else: a setup kernel that
- *     clears the work counter and, where there are more than four batches,
- *     receives their descriptors as parameters and writes them into the array,
- *     then the decode kernel, which carries up to four in its own parameters
+ *     clears the work counter and, where there are more than four batches (one
+ *     on variant 12), receives their descriptors as parameters and writes them
+ *     into the array, then the decode kernel, else with them in its parameters
  *     (both once more where variants 20 and 21 are mixed).  It can therefore be
  *     captured into a CUDA graph (after a first uncaptured call on the device);
  *     each replay decodes whatever the captured syndrome buffers hold into the

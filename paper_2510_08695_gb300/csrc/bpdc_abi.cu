@@ -596,8 +596,8 @@ int enqueue(bpdc_graph_s *g, int s, LaunchDesc &ld, int n, int64_t total, int vi
     RingSlot &rs = g->ring[s];
     cudaError_t e;
     ld.batches = nullptr;
-    if (n > kInlineBatches) {
-        for (int k = 0; k < kInlineBatches; ++k) rs.host_desc[k] = ld.own[k];
+    if (n > inline_batches(vid)) {
+        for (int k = 0; k < std::min(n, kInlineBatches); ++k) rs.host_desc[k] = ld.own[k];
         e = cudaMemcpyAsync(rs.dev_desc, rs.host_desc, sizeof(BatchDesc) * n, cudaMemcpyHostToDevice, stream);
         if (e != cudaSuccess) return cuda_fail(e, "descriptor upload");
         ld.batches = rs.dev_desc;

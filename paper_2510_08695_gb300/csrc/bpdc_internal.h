@@ -129,10 +129,18 @@ struct BatchDesc {
 // Descriptors that a launch carries in its own parameters: a request (one batch)
 // or a few need no copy to the device before the kernel.
 constexpr int kInlineBatches = 4;
+// Of variant 12 (product-sum BB codes) only one: the list form of a kernel holds a
+// pointer to descriptors that may lie in its parameters or in memory, which costs this
+// one spills of its iterations (three rates of 20000 BB[[144,12,12]] shots 7.67 -> 8.04
+// ms; 7.70 with descriptors in memory alone).  No other kernel lost more than 1 % to it.
+constexpr int inline_batches(int id) { return id == 12 ? 1 : kInlineBatches; }
+// Where a kernel finds its descriptors: in its parameters and just one, in its
+// parameters or in device memory, in device memory.
+enum DescSource { kDescOne, kDescsAnywhere, kDescsGlobal };
 
 struct LaunchDesc {
     BatchDesc own[kInlineBatches];
-    const BatchDesc *batches;    // device array of more than kInlineBatches, else null: `own`
+    const BatchDesc *batches;    // device array of more than inline_batches, else null: `own`
     int32_t n_batches;
     int64_t total;               // shots over all batches
     unsigned long long *work;    // persistent work counter, 0 before the launch and after it (nullptr: one

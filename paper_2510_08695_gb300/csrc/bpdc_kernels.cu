@@ -845,7 +845,10 @@ struct Decoder {
         }
     }
 
-    static constexpr bool kKeepPost = PVM <= 5;
+    // Not for product-sum with a lane a check: the second pair of run's instances spills
+    // registers of the first (variant 12: 50000 BB[[144,12,12]] shots at p = 0.05 5.34 ->
+    // 5.62 ms without posteriors).
+    static constexpr bool kKeepPost = PVM <= 5 && (RULE == 0 || L::kQuad);
     // One value per variable of this lane into a shot's row of posteriors.
     static __device__ __forceinline__ void write_post(const DevGraph &g, const L &ln, int u, float *post_row,
                                                       const float (&v)[PVM])
@@ -1157,19 +1160,19 @@ struct Decoder {
         }
     }
 
-    // ONE: a launch of one batch, whose descriptor is read from the kernel's
-    // parameters in place: no pointer to it is held across the iterations (the
-    // registers it takes were spilled) and a shot's fields come from the constant
-    // bank.  10^5 phenomenological BB[[72,12,6]] shots at p = 0.006 1.50 -> 1.25 ms,
-    // BB[[144,12,12]] at p = 0.002 4.49 -> 4.05 ms; distance-7 surface code 2.75 ->
+    // SRC: where the launch's descriptors lie (DescSource).  One batch: its descriptor is
+    // read from the kernel's parameters in place: no pointer to it is held across the
+    // iterations (the registers it takes were spilled) and a shot's fields come from the
+    // constant bank.  10^5 phenomenological BB[[72,12,6]] shots at p = 0.006 1.50 -> 1.23
+    // ms, BB[[144,12,12]] at p = 0.002 4.49 -> 4.03 ms; distance-7 surface code 2.75 ->
     // 2.63 ms.
-    template <bool ONE>
+    template <int SRC>
     static __device__ void decode(const LaunchDesc &ld, uint32_t *region, const Group<G> &grp, int gib)
     {
         const int u = grp.u;
-        const BatchDesc *const batches = ONE || !ld.batches ? ld.own : ld.batches;
+        const BatchDesc *const batches = SRC == kDescsAnywhere && !ld.batches ? ld.own : ld.batches;
         auto desc = [&](int i) -> const BatchDesc & {
-            if constexpr (ONE) return ld.own[0];
+            if constexpr (SRC == kDescOne) return ld.own[0];
             else return batches[i];
         };
         L ln;
@@ -1232,7 +1235,7 @@ struct Decoder {
                         for (int x = 0; x < 4; ++x) atomicAdd(desc(bi).counters + x, cnt[x]);
                     cnt[0] = cnt[1] = cnt[2] = cnt[3] = 0;
                 }
-                int lo = 0, hi = ONE ? 0 : ld.n_batches - 1;
+                int lo = 0, hi = SRC == kDescOne ? 0 : ld.n_batches - 1;
                 while (lo < hi) {  // last batch with first <= w
                     const int mid = (lo + hi + 1) >> 1;
                     if (desc(mid).first <= (int64_t)w) lo = mid; else hi = mid - 1;
@@ -1416,7 +1419,7 @@ struct Decoder {
 };
 
 template <int G, int PCM, int DCM, int PVM, int CVM, int CMIN, bool RC, int RULE, int BLOCK, int MINB,
-          uint64_t PROF, bool TAB, int TAIL, int NP, int NV, bool ONE>
+          uint64_t PROF, bool TAB, int TAIL, int NP, int NV, int SRC>
 __global__ void __launch_bounds__(BLOCK, MINB) decode_kernel(const __grid_constant__ LaunchDesc ld, int region_words)
 {
     extern __shared__ uint32_t smem[];
@@ -1435,7 +1438,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) decode_kernel(const __grid_consta
         grp.leader = 0;
     }
     uint32_t *region = smem + (size_t)gib * region_words;
-    Decoder<G, PCM, DCM, PVM, CVM, CMIN, RC, RULE, PROF, TAB, TAIL, NP, NV>::template decode<ONE>(ld, region, grp, gib);
+    Decoder<G, PCM, DCM, PVM, CVM, CMIN, RC, RULE, PROF, TAB, TAIL, NP, NV>::template decode<SRC>(ld, region, grp, gib);
 }
 
 // Cut selection alone, one block per shot (same selection code as the fused kernel).
@@ -1546,15 +1549,23 @@ bool check_status(int *, long long *) { return false; }
 // shots gain at p = 0.02 (2.83 -> 2.75 ms) but lose at 0.06 (14.75 -> 14.88 ms), where
 // the workload's time is, and BB[[72,12,6]] is 1.64 ms either way; nor those that no
 // rule chooses first (each instance costs build time).
-static constexpr bool one_batch_form(int id) { return id == 3 || id == 11 || id == 16 || id == 20 || id == 21; }
+static constexpr bool one_batch_form(int id)
+{
+    return id == 3 || id == 11 || id == 12 || id == 16 || id == 20 || id == 21;
+}
+
+// Where the instance for lists reads its descriptors.
+static constexpr int list_source(int id) { return inline_batches(id) > 1 ? kDescsAnywhere : kDescsGlobal; }
 
 static const void *variant_fn(int id, bool one)
 {
     switch (id) {
 #define X(id, G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV) \
     case id:                                                                                        \
-        return one ? (const void *)decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV, one_batch_form(id)> \
-                   : (const void *)decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV, false>;
+        return one ? (const void *)decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV, \
+                                                 one_batch_form(id) ? (int)kDescOne : list_source(id)> \
+                   : (const void *)decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV, \
+                                                 list_source(id)>;
         BPDC_VARIANTS(X)
 #undef X
     default: return nullptr;
@@ -1610,11 +1621,12 @@ cudaError_t launch_variant(int id, const LaunchDesc &ld, int grid, int groups, i
 #define X(id, G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV)                          \
     case id:                                                                                        \
         if (one)                                                                                    \
-            decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV, one_batch_form(id)> \
+            decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV,      \
+                          one_batch_form(id) ? (int)kDescOne : list_source(id)>                     \
                 <<<grid, threads, smem, s>>>(ld, region);                                           \
         else                                                                                        \
-            decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV, false>       \
-                <<<grid, threads, smem, s>>>(ld, region);                                           \
+            decode_kernel<G, PC, DC, PV, CV, CMIN, RC, RULE, BLK, MB, PROF, TAB, TAIL, NP, NV,      \
+                          list_source(id)><<<grid, threads, smem, s>>>(ld, region);                 \
         return cudaGetLastError();
         BPDC_VARIANTS(X)
 #undef X
@@ -1702,7 +1714,7 @@ cudaError_t launch_variant_static(int id, const BatchDesc *host_descs, int n, in
     ld.work = reinterpret_cast<unsigned long long *>(base);
     ld.n_batches = n;
     ld.total = total;
-    if (n <= kInlineBatches) {
+    if (n <= inline_batches(id)) {
         for (int i = 0; i < n; ++i) ld.own[i] = host_descs[i];
         static_clear_kernel<<<1, 1, 0, s>>>(ld.work);
     } else {
