@@ -219,8 +219,9 @@ typedef struct {
 } bpdc_batch;
 
 /* Decodes several batches, possibly of different graphs, in as few persistent
- * launches as the compiled kernel variants allow (one per variant), with the
- * shots of all batches of a variant behind one device work counter.  All
+ * launches as the compiled kernel variants allow (one per variant; variant 20
+ * also takes the batches of variant 21 where they are short), with the shots of
+ * all batches of a launch behind one device work counter.  All
  * graphs must live on the same device; results equal those of bpdc_decode
  * on each batch.  A launch takes at most 2^32 - 2^24 shots: longer lists are
  * split over several launches, and a single batch above that size is
@@ -270,7 +271,7 @@ int bpdc_decode_host(const bpdc_batch *batches, int32_t n_batches, int64_t chunk
  *     clears the work counter and, where there are more than four batches (one
  *     on variant 12), receives their descriptors as parameters and writes them
  *     into the array, then the decode kernel, else with them in its parameters
- *     (both once more where variants 20 and 21 are mixed).  It can therefore be
+ *     (both once more where long batches of variants 20 and 21 are mixed).  It can therefore be
  *     captured into a CUDA graph (after a first uncaptured call on the device);
  *     each replay decodes whatever the captured syndrome buffers hold into the
  *     captured output buffers.

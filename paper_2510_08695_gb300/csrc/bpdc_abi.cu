@@ -140,11 +140,13 @@ struct bpdc_graph_s {
     bpdc_opts opts{};
     HostCsr H, L, D;
     std::vector<double> priors;
+    double expected_errors = 0.0;   // sum of the priors
     DevGraph dg{};
     void *arena = nullptr;
     int variant = -1;
     int groups_per_block = 0;
     int blocks_per_sm = 0;
+    int family_bps = 0;   // residency on the variant of its family (variant_family), where that is another
     int smem_bytes = 0;
     int regs = 0;
     void *ring_mem = nullptr;
@@ -408,6 +410,11 @@ int plan_and_upload(bpdc_graph_s *g, int want_G, int want_id = -1)
     cudaError_t e = variant_attributes(vid, smem, &bps, &regs);
     if (e != cudaSuccess) return cuda_fail(e, "kernel attributes");
     if (bps < 1) return fail(BPDC_ERR_UNSUPPORTED, "kernel variant %d cannot be resident with %d bytes of shared memory", vid, smem);
+    int family_bps = 0;
+    if (variant_family(vid) != vid) {
+        e = variant_attributes(variant_family(vid), smem, &family_bps, nullptr);
+        if (e != cudaSuccess) return cuda_fail(e, "kernel attributes");
+    }
 
     // device arena
     std::vector<char> blob;
@@ -511,6 +518,7 @@ int plan_and_upload(bpdc_graph_s *g, int want_G, int want_id = -1)
     g->variant = vid;
     g->groups_per_block = gpb;
     g->blocks_per_sm = bps;
+    g->family_bps = family_bps;
     g->smem_bytes = smem;
     g->regs = regs;
     return BPDC_OK;
@@ -615,6 +623,34 @@ int enqueue(bpdc_graph_s *g, int s, LaunchDesc &ld, int n, int64_t total, int vi
     return BPDC_OK;
 }
 
+// Whether the batches of a list on a variant that specialises another one (21 of 20)
+// join that one's launch.  A launch of their own is faster by the shot but comes after
+// the other one, and the GPU drains once more: some 2 T iterations of the last shots.
+// A shot with w expected errors (the sum of its priors) takes about w^2 / 2
+// iterations, so the batches join while that work is less than what the resident
+// groups would do in kFamilyDrain T / 2 iterations each.  As many shots of
+// BB[[108,8,10]] as of BB[[144,12,12]], T = 50, two launches / one (us): p = 0.05, 64 shots
+// 89 / 70, 4000 167 / 123, 24000 341 / 320, 32000 415 / 404; p = 0.02, 24000 151 / 122;
+// p = 0.08, 4000 240 / 184, 12000 438 / 448, 24000 786 / 828.
+constexpr double kFamilyDrain = 3.0;
+bool joins_family(const bpdc_batch *batches, int n)
+{
+    int64_t own = 0;
+    double work = 0.0, drain = 0.0;
+    for (int i = 0; i < n; ++i) {
+        const bpdc_graph_s *g = batches[i].graph;
+        if (g->variant == variant_family(g->variant)) {
+            if (g->variant == variant_family(kSpecialVariant)) own += batches[i].B;
+        } else if (batches[i].B > 0) {
+            if (g->family_bps < 1) return false;
+            const double T = g->opts.max_iter, w = g->expected_errors;
+            work += (double)batches[i].B * std::min(w * w, 2.0 * T);
+            drain = std::max(drain, kFamilyDrain * T * g->sm_count * g->blocks_per_sm * g->groups_per_block);
+        }
+    }
+    return own > 0 && work <= drain;
+}
+
 int acquire_slot(bpdc_graph_s *g)
 {
     const int s = g->ring_next;
@@ -685,6 +721,7 @@ int bpdc_graph_create(const bpdc_csr *H, const bpdc_csr *L, const bpdc_csr *D, c
             return fail(BPDC_ERR_UNSUPPORTED, "row %d of D has weight above %d", r, kMaxDRowWeight);
         }
     g->priors.assign(priors, priors + N);
+    for (double p : g->priors) g->expected_errors += p;
     for (int j = 0; j < N; ++j)
         if (!(g->priors[j] > 0.0 && g->priors[j] <= 0.5)) {
             delete g;
@@ -740,11 +777,13 @@ static int replan(bpdc_graph_t g, int want_G, int want_id)
     const DevGraph keep = g->dg;
     void *keep_arena = g->arena;
     const int kv = g->variant, kg = g->groups_per_block, kb = g->blocks_per_sm, ks = g->smem_bytes;
+    const int kf = g->family_bps;
     g->arena = nullptr;
     int rc = plan_and_upload(g, want_G, want_id);
     if (rc != BPDC_OK) {
         g->dg = keep; g->arena = keep_arena; g->variant = kv;
         g->groups_per_block = kg; g->blocks_per_sm = kb; g->smem_bytes = ks;
+        g->family_bps = kf;
         return rc;
     }
     cudaFree(keep_arena);
@@ -895,19 +934,22 @@ int bpdc_decode_multi(const bpdc_batch *batches, int32_t n, void *stream)
     std::lock_guard<std::mutex> lk(owner->mu);
     DeviceGuard dgd(dev);
     // one launch per kernel variant (chunks of at most kMaxBatches batches)
+    const bool join = joins_family(batches, n);
+    auto variant_of = [&](int i) {
+        const int v = batches[i].graph->variant;
+        return join ? variant_family(v) : v;
+    };
     std::vector<int> order(n);
     for (int i = 0; i < n; ++i) order[i] = i;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-        return batches[a].graph->variant < batches[b].graph->variant;
-    });
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return variant_of(a) < variant_of(b); });
     size_t i = 0;
     while (i < order.size()) {
-        const int vid = batches[order[i]].graph->variant;
+        const int vid = variant_of(order[i]);
         const int s = acquire_slot(owner);
         int cnt = 0, smem = 0, bps = 0;
         int64_t total = 0;
         LaunchDesc ld{};
-        while (i < order.size() && cnt < kMaxBatches && batches[order[i]].graph->variant == vid) {
+        while (i < order.size() && cnt < kMaxBatches && variant_of(order[i]) == vid) {
             const bpdc_batch &bt = batches[order[i]];
             // a launch takes at most kMaxLaunchShots: the next one takes the rest
             if (cnt > 0 && total + bt.B > kMaxLaunchShots) break;
@@ -916,7 +958,7 @@ int bpdc_decode_multi(const bpdc_batch *batches, int32_t n, void *stream)
                 total += bt.B;
                 if (bt.graph->smem_bytes >= smem) {   // the widest graph bounds the residency
                     smem = bt.graph->smem_bytes;
-                    bps = bt.graph->blocks_per_sm;
+                    bps = bt.graph->variant == vid ? bt.graph->blocks_per_sm : bt.graph->family_bps;
                 }
                 ++cnt;
             }
@@ -1099,23 +1141,25 @@ int bpdc_decode_multi_noalloc(const bpdc_batch *batches, int32_t n, void *stream
     if (all > kMaxLaunchShots)
         return fail(BPDC_ERR_UNSUPPORTED, "at most %lld shots per call (got %lld)", (long long)kMaxLaunchShots,
                     (long long)all);
-    // one launch per variant of the family, in the order of the first batch of each
+    // one launch per variant, in the order of the first batch of each
+    const bool join = joins_family(batches, n);
+    auto variant_of = [&](int i) { return join ? vid : batches[i].graph->variant; };
     bool done[kStaticBatches] = {};
     for (int k = 0; k < n; ++k) {
         if (done[k] || batches[k].B == 0) continue;
-        const int id = batches[k].graph->variant;
+        const int id = variant_of(k);
         BatchDesc descs[kStaticBatches];   // host stack: no allocation
         int cnt = 0, smem = 0, bps = 0;
         int64_t total = 0;
         for (int i = k; i < n; ++i) {
             const bpdc_batch &bt = batches[i];
-            if (bt.B == 0 || bt.graph->variant != id) continue;
+            if (bt.B == 0 || variant_of(i) != id) continue;
             done[i] = true;
             fill_desc(descs[cnt], bt.graph, bt.B, bt.syndromes, bt.shot_offset, &bt.out, total);
             total += bt.B;
             if (bt.graph->smem_bytes >= smem) {
                 smem = bt.graph->smem_bytes;
-                bps = bt.graph->blocks_per_sm;
+                bps = bt.graph->variant == id ? bt.graph->blocks_per_sm : bt.graph->family_bps;
             }
             ++cnt;
         }

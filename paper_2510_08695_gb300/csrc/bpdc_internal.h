@@ -178,9 +178,12 @@ void plan_layout(int M, int N, const std::vector<int32_t> &row_ptr, const std::v
                  int npos, int dc, bool optimize, const std::vector<int> &pass_cv, Layout &out);
 
 int num_variants();
-// Variants whose graphs an allocation-free launch may mix: one and its
-// specialisation to a smaller shape (variant 21 takes graphs that 20 takes too).
-constexpr int variant_family(int id) { return id == 21 ? 20 : id; }
+// Variant 21 is variant 20 for graphs of at most two check and four variable passes.
+// Variant 20 decodes its graphs as they are packed: the slots, tables and the region of
+// a graph follow from its own passes, and the one thing that variant 20 packs in another
+// way, its shared last check pass, is the third, which these graphs do not have.
+constexpr int kSpecialVariant = 21;
+constexpr int variant_family(int id) { return id == kSpecialVariant ? 20 : id; }
 // Checked builds: the first failed bounds check since the last call (site 0:
 // none) and its index, then cleared.  Normal builds return false.
 bool check_status(int *site, long long *index);
