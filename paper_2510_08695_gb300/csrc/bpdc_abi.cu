@@ -707,9 +707,10 @@ int bpdc_graph_create(const bpdc_csr *H, const bpdc_csr *L, const bpdc_csr *D, c
     }
     const int N = g->H.cols;
     if (g->L.cols != N || g->D.cols != N) {
+        rc = fail(BPDC_ERR_DIM_MISMATCH, "H, L and D must have the same number of columns (%d, %d, %d)", N, g->L.cols,
+                  g->D.cols);
         delete g;
-        return fail(BPDC_ERR_DIM_MISMATCH, "H, L and D must have the same number of columns (%d, %d, %d)", N,
-                    g->L.cols, g->D.cols);
+        return rc;
     }
     if (N > 65535 || g->H.rows > 65535) {
         delete g;
@@ -724,8 +725,9 @@ int bpdc_graph_create(const bpdc_csr *H, const bpdc_csr *L, const bpdc_csr *D, c
     for (double p : g->priors) g->expected_errors += p;
     for (int j = 0; j < N; ++j)
         if (!(g->priors[j] > 0.0 && g->priors[j] <= 0.5)) {
+            rc = fail(BPDC_ERR_INVALID_ARG, "prior %d = %g outside (0, 1/2]", j, g->priors[j]);
             delete g;
-            return fail(BPDC_ERR_INVALID_ARG, "prior %d = %g outside (0, 1/2]", j, g->priors[j]);
+            return rc;
         }
     int ndev = 0;
     cudaError_t e = cudaGetDeviceCount(&ndev);
