@@ -1192,7 +1192,8 @@ int bpdc_sample(bpdc_graph_t g, int64_t B, uint64_t seed, uint64_t shot_offset, 
     if (B == 0) return BPDC_OK;
     if (!syndromes) return fail(BPDC_ERR_INVALID_ARG, "syndromes is NULL");
     DeviceGuard dgd(g->device);
-    cudaError_t e = launch_sample(g->dg, B, seed, shot_offset, syndromes, observables, errors, (cudaStream_t)stream);
+    cudaError_t e = launch_sample(g->dg, B, seed, shot_offset, syndromes, observables, errors, g->sm_count,
+                                  (cudaStream_t)stream);
     return e == cudaSuccess ? BPDC_OK : cuda_fail(e, "sampler launch");
 }
 
@@ -1286,6 +1287,7 @@ static int wbp_prepare(bpdc_graph_t g, int64_t B, const uint32_t *syndromes, con
         return fail(BPDC_ERR_INVALID_ARG, "workspace of %zu bytes needed", need);
     a = WbpArgs{};
     a.B = B; a.E = E; a.T = T; a.rm = rmax; a.cm = cmax; a.clip = clip;
+    a.sms = g->sm_count;
     a.syn = syndromes; a.W = weights;
     a.part = (float *)workspace;
     a.S = (float *)workspace + need / sizeof(float) - (size_t)B * T * E;

@@ -230,6 +230,7 @@ struct WbpArgs {
     int64_t B;
     int E, T;                    // edges, iterations
     int rm, cm;                  // largest row and column weight
+    int sms;                     // SMs of the device
     float clip;                  // |q| <= clip
     const uint32_t *syn;         // [B][MW]
     const float *W;              // [2][T][E]
@@ -245,6 +246,6 @@ cudaError_t launch_wbp_backward(const DevGraph &g, const WbpArgs &a, float *grad
 // runs of `reps` iterations on the current device.
 cudaError_t measure_smem_peak(int reps, double *bytes_per_s, int *num_sms);
 cudaError_t launch_sample(const DevGraph &g, int64_t B, uint64_t seed, uint64_t shot_offset,
-                          uint32_t *syn, uint32_t *obs, uint32_t *err, cudaStream_t s);
+                          uint32_t *syn, uint32_t *obs, uint32_t *err, int sms, cudaStream_t s);
 
 }  // namespace bpdc

@@ -163,15 +163,15 @@ __global__ void __launch_bounds__(kSampleThreads) sample_wide_kernel(DevGraph g,
     }
 }
 
-int grid_size(int64_t B, int per_block)
+int grid_size(int64_t B, int per_block, int sms)
 {
     const int64_t need = (B + per_block - 1) / per_block;
-    return (int)(need < 152 * 8 ? need : 152 * 8);   // 2048 threads on each of 152 SMs
+    return (int)(need < sms * 8 ? need : sms * 8);   // 2048 threads on each SM
 }
 
 template <int WARPS, int KWR>
 cudaError_t launch_wide(const DevGraph &g, int64_t B, uint64_t seed, uint64_t shot_offset, uint32_t *syn,
-                        uint32_t *obs, uint32_t *err, cudaStream_t s)
+                        uint32_t *obs, uint32_t *err, int sms, cudaStream_t s)
 {
     constexpr int TPB = kSampleThreads / 32 / WARPS;
     const size_t smem = (size_t)TPB * (g.MW + g.KW) * 4 + (size_t)8 * ((g.NW + WARPS - 1) / WARPS) * 32 * 2;
@@ -181,14 +181,14 @@ cudaError_t launch_wide(const DevGraph &g, int64_t B, uint64_t seed, uint64_t sh
         if (e != cudaSuccess) return e;
     }
     sample_wide_kernel<WARPS, KWR>
-        <<<grid_size(B, TPB), kSampleThreads, smem, s>>>(g, B, seed, shot_offset, syn, obs, err);
+        <<<grid_size(B, TPB, sms), kSampleThreads, smem, s>>>(g, B, seed, shot_offset, syn, obs, err);
     return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_sample(const DevGraph &g, int64_t B, uint64_t seed, uint64_t shot_offset, uint32_t *syn,
-                          uint32_t *obs, uint32_t *err, cudaStream_t s)
+                          uint32_t *obs, uint32_t *err, int sms, cudaStream_t s)
 {
     if (B <= 0) return cudaSuccess;
     if (g.NW <= kSampleMaskWords && g.MW + g.KW <= 32) {
@@ -196,11 +196,11 @@ cudaError_t launch_sample(const DevGraph &g, int64_t B, uint64_t seed, uint64_t 
         decltype(&sample_narrow_kernel<1>) const fn[] = {
             sample_narrow_kernel<1>, sample_narrow_kernel<2>, sample_narrow_kernel<3>, sample_narrow_kernel<4>,
             sample_narrow_kernel<5>, sample_narrow_kernel<6>, sample_narrow_kernel<7>, sample_narrow_kernel<8>};
-        fn[g.NW - 1]<<<grid_size(B, 8), kSampleThreads, 0, s>>>(g, B, seed, shot_offset, syn, obs, err);
+        fn[g.NW - 1]<<<grid_size(B, 8, sms), kSampleThreads, 0, s>>>(g, B, seed, shot_offset, syn, obs, err);
         return cudaGetLastError();
     }
     auto go = [&](auto w, auto k) {
-        return launch_wide<decltype(w)::value, decltype(k)::value>(g, B, seed, shot_offset, syn, obs, err, s);
+        return launch_wide<decltype(w)::value, decltype(k)::value>(g, B, seed, shot_offset, syn, obs, err, sms, s);
     };
     using std::integral_constant;
     // a block per shot also where eight shots' logical words would not fit its memory

@@ -343,9 +343,9 @@ __global__ void __launch_bounds__(256) wbp_reduce_kernel(const float *part, int 
 // shots 195 / 237 against 182 / 186; 300 shots 168 / 214 against 124 / 169.
 // Phenomenological BB[[72,12,6]] (1944 edges, 7 shots fit an SM), 3000 shots, T = 6:
 // 438 / 1134 against 360 / 615.
-int team_size(int64_t B, int E)
+int team_size(int64_t B, int E, int sms)
 {
-    const int64_t per_sm = std::min<int64_t>((B + 151) / 152, (int64_t)(kMaxWbpSmem / ((size_t)16 * E)));
+    const int64_t per_sm = std::min<int64_t>((B + sms - 1) / sms, (int64_t)(kMaxWbpSmem / ((size_t)16 * E)));
     return per_sm * 2 >= 16 ? 64 : 256;
 }
 
@@ -355,12 +355,12 @@ int team_size(int64_t B, int E)
 // 4 blocks do not fit an SM: the teams' named barriers take all 16 of a block, and
 // an SM has 64 (blocks of 3 shots, 27 on an SM, ran 12 at a time: forward 406 us
 // against 328).
-int shots_per_block(int64_t B, int least, int most)
+int shots_per_block(int64_t B, int least, int most, int sms)
 {
     int best = most;
     int64_t load = INT64_MAX;
     for (int w = most; w >= least; --w) {
-        const int64_t n = ((B + w - 1) / w + 151) / 152;
+        const int64_t n = ((B + w - 1) / w + sms - 1) / sms;
         if (n > 4 && w < most) break;
         if (n * w < load) { best = w; load = n * w; }
     }
@@ -371,11 +371,11 @@ int shots_per_block(int64_t B, int least, int most)
 // floats a block) lie before the saved S in the workspace, which leaves at least
 // B (T + 1) E floats: at least four shots a block, and blocks take several rounds of
 // shots where that is short.
-void backward_plan(int64_t B, int E, int T, int G, int *shots, int64_t *blocks)
+void backward_plan(int64_t B, int E, int T, int G, int sms, int *shots, int64_t *blocks)
 {
     const int most = (int)std::min<size_t>(most_shots(G), kMaxWbpSmem / ((size_t)16 * E));
     const int64_t room = std::max<int64_t>(1, B * (T + 1) / ((int64_t)4 * T));
-    int w = shots_per_block(B, std::min(4, most), most);
+    int w = shots_per_block(B, std::min(4, most), most, sms);
     while (w < most && (B + w - 1) / w > room) ++w;
     *shots = (int)std::min<int64_t>(w, B);
     *blocks = std::min((B + *shots - 1) / *shots, room);
@@ -394,10 +394,10 @@ cudaError_t launch_wbp_forward(const DevGraph &g, const WbpArgs &a, cudaStream_t
 {
     if (a.B <= 0) return cudaSuccess;
     if (a.E > kWbpMaxEdges) return cudaErrorInvalidValue;
-    const int G = team_size(a.B, a.E);
-    const int w = shots_per_block(a.B, 1, most_shots(G));
+    const int G = team_size(a.B, a.E, a.sms);
+    const int w = shots_per_block(a.B, 1, most_shots(G), a.sms);
     const size_t smem = (size_t)w * a.E * sizeof(float);
-    const int grid = (int)std::min<int64_t>((a.B + w - 1) / w, 152 * 32);
+    const int grid = (int)std::min<int64_t>((a.B + w - 1) / w, (int64_t)a.sms * 32);
     auto go = [&](auto kernel) {
         const cudaError_t e = allow_smem(kernel, smem);
         if (e != cudaSuccess) return e;
@@ -414,10 +414,10 @@ cudaError_t launch_wbp_backward(const DevGraph &g, const WbpArgs &a, float *grad
     const int64_t n = (int64_t)2 * a.T * a.E;
     if (a.B <= 0) return cudaMemsetAsync(grad_w, 0, sizeof(float) * n, s);
     if (a.E > kWbpMaxEdges) return cudaErrorInvalidValue;
-    const int G = team_size(a.B, a.E);
+    const int G = team_size(a.B, a.E, a.sms);
     int w;
     int64_t blocks;
-    backward_plan(a.B, a.E, a.T, G, &w, &blocks);
+    backward_plan(a.B, a.E, a.T, G, a.sms, &w, &blocks);
     const size_t smem = (size_t)w * 4 * a.E * sizeof(float);
     auto go = [&](auto kernel) {
         const cudaError_t e = allow_smem(kernel, smem);
