@@ -826,21 +826,16 @@ struct Decoder {
         }
     }
 
-    // The check passes P .. END-1 of the fast path, NP at a time; lanes without a
-    // check in the variant's last pass skip it.
+    // The check passes P .. END-1 of the fast path, NP at a time; every lane has a
+    // check in each (the variant's last pass, where some have none, is a shared one).
     template <int P, int END>
     static __device__ __forceinline__ void held_passes(const L &ln, uint32_t sbits, float alpha, bool scatter,
                                                        uint32_t &unsat)
     {
+        static_assert(TAIL > 0, "passes are grouped before a shared last pass");
         if constexpr (P < END) {
             constexpr int N = (END - P < NP) ? (END - P) : NP;
-            if constexpr (P + N < PCM) {
-                held_rows<P, N>(ln, sbits, alpha, scatter, unsat);
-            } else if ((ln.cvalid >> (PCM - 1)) & 1u) {
-                held_rows<P, N>(ln, sbits, alpha, scatter, unsat);
-            } else if constexpr (N > 1) {
-                held_rows<P, N - 1>(ln, sbits, alpha, scatter, unsat);
-            }
+            held_rows<P, N>(ln, sbits, alpha, scatter, unsat);
             held_passes<P + N, END>(ln, sbits, alpha, scatter, unsat);
         }
     }
@@ -901,9 +896,9 @@ struct Decoder {
             if constexpr (L::kQuad) unsat = quad_checks(g, ln, u, t, sbits, scatter);
             if constexpr (kGroup) {
                 float qt[kTailEdges];   // the shared last pass is gathered before the others scatter
-                if constexpr (TAIL > 0) tail_gather(ln, PCM - 1, qt);
-                held_passes<0, (TAIL > 0 ? PCM - 1 : PCM)>(ln, sbits, alpha, scatter, unsat);
-                if constexpr (TAIL > 0) unsat |= tail_pass(ln, PCM - 1, sbits, alpha, scatter, qt);
+                tail_gather(ln, PCM - 1, qt);
+                held_passes<0, PCM - 1>(ln, sbits, alpha, scatter, unsat);
+                unsat |= tail_pass(ln, PCM - 1, sbits, alpha, scatter, qt);
             }
 #pragma unroll
             for (int p = 0; p < (L::kQuad || kGroup ? 0 : PCM); ++p) {
