@@ -32,7 +32,7 @@
 // to beyond the float range.  A store of every shot's gradients was 283 MB a call.
 //
 // BB[[144,12,12]], T = 20, 4096 shots: forward 545 -> 299 us (issue 79 %), adjoint
-// with the sum of the gradients 3330 -> 565 us a call (11 900 -> about 5050 warp
+// with the sum of the gradients 3310 -> 567 us a call (11 900 -> about 5050 warp
 // instructions per shot and iteration).
 #include <cuda_runtime.h>
 
@@ -75,7 +75,7 @@ __device__ __forceinline__ void team_sync(int team)
 // float that collects the sum, one that collects its exact rounding errors (two-sum)
 // and one for theirs, added up in FP64 at the end.  FP64 runs at a 64th of the FP32
 // rate here: with an FP64 add for each of the 71 million terms of 4096 BB[[144,12,12]]
-// shots, T = 20, a backward call takes 599 us, with this form 565 (533 with two floats,
+// shots, T = 20, a backward call takes 599 us, with this form 567 (533 with two floats,
 // some 48 bits and the range of one).  Sums that leave the float range on the way, or
 // hold an infinity or a NaN, are taken again term by term in FP64.
 __device__ __forceinline__ void two_sum(float &s, float x, float &err)
@@ -83,6 +83,19 @@ __device__ __forceinline__ void two_sum(float &s, float x, float &err)
     const float t = s + x, b = t - s;
     err = (s - (t - b)) + (x - b);
     s = t;
+}
+// Conversions to FP64 run at that rate too, so the three floats are widened by integer
+// operations (zero and normal ones; a sum with a denormal goes term by term as well):
+// 3000 phenomenological BB[[72,12,6]] shots, T = 6, 762 -> 679 us (610 with two floats).
+__device__ __forceinline__ bool zero_or_normal(float x)
+{
+    return (__float_as_uint(x) & 0x7FFFFFFFu) - 1u >= 0x007FFFFFu;
+}
+__device__ __forceinline__ double widen(float x)
+{
+    const uint32_t u = __float_as_uint(x), m = u & 0x7FFFFFFFu;
+    const uint32_t hi = m ? (m >> 3) + ((1023u - 127u) << 20) : 0u;
+    return __hiloint2double((int)((u & 0x80000000u) | hi), (int)(u << 29));
 }
 template <int MOST>
 __device__ __forceinline__ double sum64(const float *x, int n, size_t stride)
@@ -101,7 +114,8 @@ __device__ __forceinline__ double sum64(const float *x, int n, size_t stride)
         c += f;
     }
     // where a is not finite, neither is its error b
-    if (isfinite(b + c)) return (double)a + ((double)b + (double)c);
+    if (isfinite(b + c) && zero_or_normal(a) && zero_or_normal(b) && zero_or_normal(c))
+        return widen(a) + (widen(b) + widen(c));
     double s = 0.0;
     for (int w = 0; w < n; ++w) s += (double)x[w * stride];
     return s;
@@ -339,10 +353,10 @@ __global__ void __launch_bounds__(256) wbp_reduce_kernel(const float *part, int 
 
 // Threads per shot: 64 where that gives every SM 16 warps (of the shots an SM gets
 // and has memory for in the adjoint), else 256.  BB[[144,12,12]], T = 20, forward /
-// backward call: 2000 shots 236 / 328 us with 64 threads, 293 / 349 with 256; 1023
-// shots 195 / 237 against 182 / 186; 300 shots 168 / 214 against 124 / 169.
+// backward call: 2000 shots 220 / 315 us with 64 threads, 288 / 380 with 256; 1023
+// shots 188 / 243 against 177 / 204; 300 shots 170 / 227 against 123 / 172.
 // Phenomenological BB[[72,12,6]] (1944 edges, 7 shots fit an SM), 3000 shots, T = 6:
-// 438 / 1134 against 360 / 615.
+// 367 / 1428 against 348 / 679.
 int team_size(int64_t B, int E, int sms)
 {
     const int64_t per_sm = std::min<int64_t>((B + sms - 1) / sms, (int64_t)(kMaxWbpSmem / ((size_t)16 * E)));
@@ -351,7 +365,7 @@ int team_size(int64_t B, int E, int sms)
 
 // Shots of a block (at most `most`) for an even load: the SM with the most blocks
 // gets as few shots as possible, then the most shots a block.  4096 shots take 4
-// blocks of 7 on an SM instead of 4 of 8 (adjoint 586 -> 502 us with it).  More than
+// blocks of 7 on an SM instead of 4 of 8 (backward call 599 -> 567 us).  More than
 // 4 blocks do not fit an SM: the teams' named barriers take all 16 of a block, and
 // an SM has 64 (blocks of 3 shots, 27 on an SM, ran 12 at a time: forward 406 us
 // against 328).
