@@ -586,8 +586,9 @@ void fill_desc(BatchDesc &d, const bpdc_graph_s *g, int64_t B, const uint32_t *s
     d.cut_in = o->cut_in;
 }
 
-// Descriptors of a launch on ring slot rs: up to kInlineBatches travel with the
-// launch (ld), more in the slot's pinned mirror.
+// Descriptors of a launch on ring slot rs: the first kInlineBatches are written into
+// the launch (ld), more into the slot's pinned mirror; enqueue puts a list that does
+// not travel with its launch (inline_batches) together there.
 BatchDesc *desc_of(LaunchDesc &ld, const RingSlot &rs, int k) { return k < kInlineBatches ? &ld.own[k] : &rs.host_desc[k]; }
 
 // Enqueues one launch of variant `vid` over the n descriptors written by desc_of

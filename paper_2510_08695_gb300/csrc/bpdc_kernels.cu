@@ -257,9 +257,10 @@ __device__ __forceinline__ float fmax3_abs(float a, float b, float c)
 // magnitude take one instruction each, and the middle one is what is left of
 // their XOR (needed anyway, for the parities) without m and M, up to the sign:
 // 7.5 instructions for three edges where pairs take 9 (the ALU pipe is the first
-// bound of the check update).  Exact in any order.  2-5 % of a decode: HGP-2500 p =
+// bound of the check update).  Exact in any order.  2-3 % of a decode: HGP-2500 p =
 // 0.06, 20000 shots 10.18 -> 9.97 ms; BB[[144,12,12]] p = 0.08, 10^5 shots 1.81 ->
-// 1.76 ms; phenomenological p = 0.006, 10^5 shots 9.02 -> 8.56 ms.
+// 1.76 ms; the phenomenological model's time is in its last shots, where it gains
+// nothing outside the spread (10^5 shots at p = 0.006).
 struct RowMin {
     float mn1, mn2;
     uint32_t S;   // bit 31: sign parity, bit 0: hard-decision parity
