@@ -377,8 +377,8 @@ int bpdc_wbp_forward(bpdc_graph_t g, int64_t B, const uint32_t *syndromes, const
                      void *stream);
 
 /* Adjoint: given dLoss/dL_j(t) (device float [B][T][N]), writes
- * dLoss/dW (device float [2][T][E], summed over the B shots in a fixed
- * order, so the result is deterministic). */
+ * dLoss/dW (device float [2][T][E], summed over the B shots in FP64 in a
+ * fixed order, so the result is deterministic). */
 int bpdc_decode_backward(bpdc_graph_t g, int64_t B, const uint32_t *syndromes, const float *weights, int32_t T,
                          float clip, int32_t ckpt_every, const float *grad_posteriors, float *grad_weights,
                          void *workspace, size_t workspace_bytes, void *stream);
